@@ -241,7 +241,7 @@ struct ExactDesc {
 };
 struct DirectDesc {
     int mode, n_chan, n_scan, n_f, nx, ny, nz;
-    int uniform;                    // evenly spaced band: rotation from k_0 by dk
+    int uniform;                    // evenly spaced band: polynomial in e^{j dk R}
     double x0, dx, y0, dy, z0, dz;
     float k0_hi, k0_lo, dk_hi, dk_lo;
 };

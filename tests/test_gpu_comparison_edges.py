@@ -52,6 +52,23 @@ def rel(a, b):
 
 
 @pytest.mark.parametrize("kw", [
+    dict(n_f=2, n_scan=33, n_pad=33), dict(n_f=16, n_scan=1, n_pad=1), dict(n_f=512),
+    dict(n_f=530, mode=1), dict(nx=43, ny=3, nz=1), dict(nx=127, ny=1, mode=1),
+    dict(n_f=33, n_scan=19, n_pad=20)],
+    ids=lambda kw: "-".join("%s%d" % kv for kv in kw.items()))
+def test_direct_bp_edges(binding, kw):
+    w = workload(**kw)
+    e = echo_of(w)
+    img = binding.Plan.from_workload(w).execute_bp_direct(torch.from_numpy(e).cuda()).cpu().numpy()
+    zz, yy, xx = np.meshgrid(w.axis("z"), w.axis("y"), w.axis("x"), indexing="ij")
+    ref = oracle.bp_direct(w.tx_xy, w.rx_xy, e, w.z_scan, w.f_hz,
+                           np.stack([xx.ravel(), yy.ravel(), zz.ravel()], 1))
+    err = rel(img.ravel(), ref)
+    print("direct BP %s: rel L2 %.3e" % (kw, err))
+    assert err < TOL
+
+
+@pytest.mark.parametrize("kw", [
     dict(n_scan=5, n_pad=7), dict(n_f=256), dict(n_f=257, mode=1), dict(n_f=1),
     dict(nx=17, ny=9), dict(nx=33, ny=1, mode=1), dict(dx=0.0102),
     dict(dx=0.05, f1=28.02e9), dict(dx=0.05, mode=1, n_f=257, f1=28.02e9),
