@@ -20,9 +20,7 @@
 // an element gather otherwise) and the B tile in shared memory.
 // The backward pass reuses the forward kernel for the input gradient (the
 // transposed convolution is a convolution with flipped taps and swapped
-// channel roles) and has its own GEMM for the weight gradient, reducing over
-// voxels in chunks: each chunk writes its partial dW, and a second kernel sums
-// the partials in chunk order, so gradients are bitwise reproducible.
+// channel roles); the weight gradient is in nn_wgrad.cu.
 #include <cuda_bf16.h>
 
 #include "common.cuh"
@@ -146,90 +144,6 @@ k_conv3d(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__restrict__ 
             }
         }
     }
-}
-
-// gw[co][k] += sum_v gy[v][co] x~[v][k]  (k < 27 Cin), over a chunk of voxels.
-// Block: 4 warps, 32 k-columns (8 per warp), all Cout (MT m-tiles of 16).
-template <int MT>
-__global__ void __launch_bounds__(128)
-k_conv3d_wgrad(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__restrict__ gy,
-               float *__restrict__ part, Vol vol, int Cin, int Cout, int Kp, int chunk) {
-    __shared__ __align__(16) __nv_bfloat16 As[16 * MT][kRowPad];   // [co][16 voxels]
-    __shared__ __align__(16) __nv_bfloat16 Bs[32][kRowPad];        // [k col][16 voxels]
-    const int V = vol.D * vol.H * vol.W;
-    const int K = 27 * Cin;
-    const int kc0 = blockIdx.x * 32;
-    const int vbeg = blockIdx.y * chunk;
-    const int vend = min(V, vbeg + chunk);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int g = lane >> 2, t = lane & 3;
-    float acc[MT][4];
-#pragma unroll
-    for (int i = 0; i < MT; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
-    for (int vs = vbeg; vs < vend; vs += 16) {
-        for (int e = threadIdx.x; e < 16 * 16 * MT; e += 128) {
-            const int vv = e / (16 * MT), co = e - vv * (16 * MT);
-            const int v = vs + vv;
-            As[co][vv] = (v < vend && co < Cout) ? gy[(size_t)v * Cout + co] : __float2bfloat16(0.f);
-        }
-        for (int e = threadIdx.x; e < 32 * 16; e += 128) {
-            const int kc = e >> 4, vv = e & 15;
-            const int k = kc0 + kc, v = vs + vv;
-            __nv_bfloat16 val = __float2bfloat16(0.f);
-            int nv;
-            if (v < vend && k < K) {
-                const int tap = k / Cin, ci = k - tap * Cin;
-                if (vol.neighbour(v, tap, nv)) val = x[(size_t)nv * Cin + ci];
-            }
-            Bs[kc][vv] = val;
-        }
-        __syncthreads();
-        unsigned b[2];
-        b[0] = ld_pair(&Bs[warp * 8 + g][2 * t]);
-        b[1] = ld_pair(&Bs[warp * 8 + g][2 * t + 8]);
-#pragma unroll
-        for (int i = 0; i < MT; ++i) {
-            unsigned a[4];
-            a[0] = ld_pair(&As[i * 16 + g][2 * t]);
-            a[1] = ld_pair(&As[i * 16 + g + 8][2 * t]);
-            a[2] = ld_pair(&As[i * 16 + g][2 * t + 8]);
-            a[3] = ld_pair(&As[i * 16 + g + 8][2 * t + 8]);
-            mma_bf16_16816(acc[i], a, b);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int i = 0; i < MT; ++i)
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                const int co = i * 16 + g + 8 * h;
-                const int k = kc0 + warp * 8 + 2 * t + q;
-                if (co < Cout && k < K)
-                    part[((size_t)blockIdx.y * Cout + co) * Kp + k] = acc[i][2 * h + q];
-            }
-}
-
-// gw[i] += sum_c part[c][i] in chunk order (deterministic)
-__global__ void k_sum_parts(const float *__restrict__ part, float *__restrict__ gw, int nparts,
-                            size_t n) {
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float s = 0.f;
-    for (int c = 0; c < nparts; ++c) s += part[(size_t)c * n + i];
-    gw[i] += s;
-}
-
-// part[chunk][co] = sum over the chunk's voxels of gy[v][co]
-__global__ void k_bias_grad(const __nv_bfloat16 *__restrict__ gy, float *__restrict__ part, int V,
-                            int C, int chunk) {
-    const int co = threadIdx.x;
-    if (co >= C) return;
-    const int v0 = blockIdx.x * chunk, v1 = min(V, v0 + chunk);
-    float s = 0.f;
-    for (int v = v0; v < v1; ++v) s += __bfloat162float(gy[(size_t)v * C + co]);
-    part[(size_t)blockIdx.x * C + co] = s;
 }
 
 // wt[ci][tap' Cout + co] = w[co][tap Cin + ci], tap' = 26 - tap
@@ -523,45 +437,6 @@ cudaError_t nn_conv3d(const void *x, const void *w, const float *bias, void *out
         dim3 grid((V + 63) / 64, (Cout + 31) / 32);
         if (out_bf16) k_conv3d<4, true><<<grid, 128, 0, st>>>(xb, wb, bias, out, vol, Cin, Cout, Kp, relu);
         else k_conv3d<4, false><<<grid, 128, 0, st>>>(xb, wb, bias, out, vol, Cin, Cout, Kp, relu);
-    }
-    return cudaGetLastError();
-}
-
-size_t nn_wgrad_work_floats(int D, int H, int W, int Cin, int Cout, int Kp) {
-    const int V = D * H * W;
-    const size_t chunks = (size_t)(V + 2047) / 2048;
-    const size_t bchunks = (size_t)(V + 4095) / 4096;
-    return chunks * Cout * Kp + bchunks * Cout;
-}
-
-cudaError_t nn_conv3d_wgrad(const void *x, const void *gy, float *gw, float *gb, float *work,
-                            int D, int H, int W, int Cin, int Cout, int Kp, cudaStream_t st) {
-    const int V = D * H * W;
-    Vol vol{D, H, W};
-    const int chunk = 2048;
-    const int nch = (V + chunk - 1) / chunk;
-    dim3 grid((27 * Cin + 31) / 32, nch);
-    const auto *xb = (const __nv_bfloat16 *)x;
-    const auto *gyb = (const __nv_bfloat16 *)gy;
-    const int mt = (Cout + 15) / 16;
-    // partials [chunk][Cout][Kp]; columns k >= 27 Cin stay zero
-    cudaError_t e = cudaMemsetAsync(work, 0, sizeof(float) * (size_t)nch * Cout * Kp, st);
-    if (e != cudaSuccess) return e;
-    switch (mt) {
-        case 1: k_conv3d_wgrad<1><<<grid, 128, 0, st>>>(xb, gyb, work, vol, Cin, Cout, Kp, chunk); break;
-        case 2: k_conv3d_wgrad<2><<<grid, 128, 0, st>>>(xb, gyb, work, vol, Cin, Cout, Kp, chunk); break;
-        case 4: k_conv3d_wgrad<4><<<grid, 128, 0, st>>>(xb, gyb, work, vol, Cin, Cout, Kp, chunk); break;
-        case 8: k_conv3d_wgrad<8><<<grid, 128, 0, st>>>(xb, gyb, work, vol, Cin, Cout, Kp, chunk); break;
-        default: return cudaErrorInvalidValue;
-    }
-    const size_t nw = (size_t)Cout * Kp;
-    k_sum_parts<<<nblk(nw), 256, 0, st>>>(work, gw, nch, nw);
-    if (gb) {
-        const int bchunk = 4096;
-        const int nb = (V + bchunk - 1) / bchunk;
-        float *bpart = work + (size_t)nch * Cout * Kp;
-        k_bias_grad<<<nb, ((Cout + 31) / 32) * 32, 0, st>>>(gyb, bpart, V, Cout, bchunk);
-        k_sum_parts<<<nblk(Cout), 256, 0, st>>>(bpart, gb, nb, Cout);
     }
     return cudaGetLastError();
 }
