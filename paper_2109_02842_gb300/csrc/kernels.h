@@ -275,6 +275,11 @@ cudaError_t launch_synth_echo(int n_chan, const double *tx_xy, const double *rx_
 cudaError_t nn_conv3d_mma(const void *x, const void *w, const float *bias, void *out, int D, int H,
                           int W, int Cin, int Cout, int Kp, int relu, int out_bf16, cudaStream_t st);
 
+// ---- nn_conv_small.cu: the convolution of one to four input channels ------------
+// cudaErrorNotSupported (nothing launched) for the shapes it does not take
+cudaError_t nn_conv3d_small(const void *x, const void *w, const float *bias, void *out, int D, int H,
+                            int W, int Cin, int Cout, int Kp, int relu, int out_bf16, cudaStream_t st);
+
 // ---- nn_tc.cu: the convolution on the tensor cores (tcgen05) -------------------
 bool nn_conv3d_tc_supported(int D, int H, int W, int Cin, int Cout, const void *x, const void *w,
                             const void *out);

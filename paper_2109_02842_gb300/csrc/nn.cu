@@ -10,9 +10,10 @@
 //
 // The convolution is an implicit GEMM on the tensor cores: out[v][co] =
 // sum_k A[v][k] B[k][co] with A the (never materialised) im2col matrix and B
-// the weights. Cin a multiple of 16 takes nn_conv_mma.cu or, wide and in
-// shapes that suit it, the tcgen05 kernel of nn_tc.cu; what those refuse (the
-// 3-channel input layer, other Cin, unaligned operands) the kernel below, BF16 mma.sync m16n8k16 with FP32 accumulation. All sum in the same
+// the weights. Cin of one to four takes nn_conv_small.cu, Cin a multiple of 16
+// nn_conv_mma.cu or, wide and in shapes that suit it, the tcgen05 kernel of
+// nn_tc.cu; what those refuse (other Cin, unaligned operands) the kernel
+// below, BF16 mma.sync m16n8k16 with FP32 accumulation. All sum in the same
 // order, K in steps of 16, with equal results bit for bit. A block of 4
 // warps owns 64 voxels x (8 NT) output channels; per 16-wide K chunk it
 // stages the A tile (one 32-byte row per voxel when Cin is a multiple of 16,
@@ -417,6 +418,9 @@ inline unsigned nblk(size_t n, int t = 256) { return (unsigned)((n + t - 1) / t)
 // ---------------------------------------------------------------------------
 cudaError_t nn_conv3d(const void *x, const void *w, const float *bias, void *out, int D, int H,
                       int W, int Cin, int Cout, int Kp, int relu, int out_bf16, cudaStream_t st) {
+    // one to four channels: the gathering column kernel
+    cudaError_t e = nn_conv3d_small(x, w, bias, out, D, H, W, Cin, Cout, Kp, relu, out_bf16, st);
+    if (e != cudaErrorNotSupported) return e;
     // wide layers of many tiles of 128 voxels: the tcgen05 kernel. Measured
     // both ways (us, tcgen05 / mma.sync columns): 64 -> 32 on 1536 tiles 133 /
     // 171, 64 -> 128 on 192 tiles 42 / 64; but 64 -> 64 on 192 tiles 39 / 35,
@@ -426,7 +430,7 @@ cudaError_t nn_conv3d(const void *x, const void *w, const float *bias, void *out
     const bool wide = Cin >= 64 && (long long)D * H * W / 128 * Cout >= 16384;
     const bool tc = nn_conv3d_tc_supported(D, H, W, Cin, Cout, x, w, out);
     if (!(wide && tc)) {
-        const cudaError_t e = nn_conv3d_mma(x, w, bias, out, D, H, W, Cin, Cout, Kp, relu, out_bf16, st);
+        e = nn_conv3d_mma(x, w, bias, out, D, H, W, Cin, Cout, Kp, relu, out_bf16, st);
         if (e != cudaErrorNotSupported) return e;
     }
     if (tc) return nn_conv3d_tc(x, w, bias, out, D, H, W, Cin, Cout, Kp, relu, out_bf16, st);

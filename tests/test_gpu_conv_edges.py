@@ -38,7 +38,9 @@ def reference(x, w, b, dims, cin):
     ((3, 2, 129), 16, 15), ((2, 6, 160), 32, 32), ((2, 3, 260), 16, 48), ((40, 33, 24), 16, 16),
     ((7, 40, 16), 64, 32), ((5, 9, 32), 64, 64), ((3, 7, 33), 32, 64), ((4, 18, 16), 64, 128),
     ((3, 5, 20), 48, 80), ((2, 16, 16), 128, 64), ((2, 5, 9), 128, 32), ((2, 3, 5), 96, 20),
-    ((160, 2, 6), 16, 16), ((3, 70, 3), 32, 32)])
+    ((160, 2, 6), 16, 16), ((3, 70, 3), 32, 32),
+    ((1, 1, 1), 3, 16), ((9, 10, 13), 1, 2), ((3, 33, 81), 3, 16), ((17, 5, 128), 2, 16),
+    ((2, 300, 1), 4, 33), ((5, 3, 170), 3, 9), ((4, 7, 6), 5, 16)])
 def test_conv_edges(L, dims, cin, cout):
     g = torch.Generator(device="cuda").manual_seed(dims[2] * 1000 + cin)
     v = dims[0] * dims[1] * dims[2]
