@@ -160,22 +160,68 @@ __global__ void k_weight_flip(const __nv_bfloat16 *__restrict__ w, __nv_bfloat16
     wt[idx] = v;
 }
 
-// out (bf16) = g (f32) where y > 0, else 0
-__global__ void k_relu_bwd(const float *__restrict__ g, const __nv_bfloat16 *__restrict__ y,
-                           __nv_bfloat16 *__restrict__ out, size_t n) {
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = __float2bfloat16(__bfloat162float(y[i]) > 0.f ? g[i] : 0.f);
+// The element-wise passes are bound by memory. Eight elements (16 bytes of
+// BF16) a thread where every operand is 16-byte aligned, the rest one by one:
+// 25 M elements, ReLU backward 0.099 -> 0.027 ms, sum 0.064 -> 0.021 ms (200
+// and 150 MB; one element a thread kept too few bytes in flight).
+struct bf8 {
+    uint4 q;
+    __device__ __forceinline__ float get(int i) const {
+        const unsigned w = i < 2 ? q.x : i < 4 ? q.y : i < 6 ? q.z : q.w;
+        return __uint_as_float((i & 1) ? (w & 0xffff0000u) : (w << 16));
+    }
+    __device__ static __forceinline__ bf8 of(const float (&f)[8]) {
+        unsigned w[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            __nv_bfloat162 h = __floats2bfloat162_rn(f[2 * k], f[2 * k + 1]);
+            w[k] = *reinterpret_cast<unsigned *>(&h);
+        }
+        return {make_uint4(w[0], w[1], w[2], w[3])};
+    }
+};
+__device__ __forceinline__ void load8(const float *p, float (&f)[8]) {
+    const float4 a = reinterpret_cast<const float4 *>(p)[0], b = reinterpret_cast<const float4 *>(p)[1];
+    f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w;
+    f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
+}
+__device__ __forceinline__ bf8 load8(const __nv_bfloat16 *p) {
+    return {*reinterpret_cast<const uint4 *>(p)};
 }
 
-__global__ void k_cast_bf16(const float *__restrict__ a, __nv_bfloat16 *__restrict__ out, size_t n) {
+// OP 0: out (bf16) = g (f32) where y > 0, else 0; 1: out (bf16) = g; 2: out
+// (bf16) = a + b (bf16). n8 groups of eight elements, then up to n.
+template <int OP>
+__global__ void __launch_bounds__(256)
+k_to_bf16(const void *__restrict__ a, const __nv_bfloat16 *__restrict__ b,
+          __nv_bfloat16 *__restrict__ out, size_t n8, size_t n) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = __float2bfloat16(a[i]);
-}
-
-__global__ void k_add_bf16(const __nv_bfloat16 *__restrict__ a, const __nv_bfloat16 *__restrict__ b,
-                           __nv_bfloat16 *__restrict__ out, size_t n) {
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = __float2bfloat16(__bfloat162float(a[i]) + __bfloat162float(b[i]));
+    const float *af = (const float *)a;
+    const __nv_bfloat16 *ab = (const __nv_bfloat16 *)a;
+    if (i < n8) {
+        float f[8];
+        if (OP == 2) {
+            const bf8 p = load8(ab + 8 * i), q = load8(b + 8 * i);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) f[k] = p.get(k) + q.get(k);
+        } else {
+            load8(af + 8 * i, f);
+            if (OP == 0) {
+                const bf8 y = load8(b + 8 * i);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) f[k] = y.get(k) > 0.f ? f[k] : 0.f;
+            }
+        }
+        *reinterpret_cast<uint4 *>(out + 8 * i) = bf8::of(f).q;
+        return;
+    }
+    const size_t e = 8 * n8 + (i - n8);
+    if (e >= n) return;
+    float f;
+    if (OP == 0) f = __bfloat162float(b[e]) > 0.f ? af[e] : 0.f;
+    else if (OP == 1) f = af[e];
+    else f = __bfloat162float(ab[e]) + __bfloat162float(b[e]);
+    out[e] = __float2bfloat16(f);
 }
 
 __global__ void k_accum_f32(const float *__restrict__ a, float *__restrict__ acc, size_t n) {
@@ -198,6 +244,28 @@ __global__ void k_avgpool2(const __nv_bfloat16 *__restrict__ x, __nv_bfloat16 *_
         s += __bfloat162float(x[(((size_t)z * H + yy) * W + xx) * C + c]);
     }
     y[i] = __float2bfloat16(0.125f * s);
+}
+
+// the same with 8 channels (16 bytes) per thread, for C a multiple of 8
+__global__ void k_avgpool2_v8(const __nv_bfloat16 *__restrict__ x, __nv_bfloat16 *__restrict__ y,
+                              int D, int H, int W, int C8) {
+    const size_t n = (size_t)(D / 2) * (H / 2) * (W / 2) * C8;
+    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int c = (int)(i % C8);
+    const size_t o = i / C8;
+    const int X = (int)(o % (W / 2)), Y = (int)((o / (W / 2)) % (H / 2)), Z = (int)(o / ((W / 2) * (H / 2)));
+    float s[8] = {};
+#pragma unroll
+    for (int d = 0; d < 8; ++d) {
+        const int z = 2 * Z + (d >> 2), yy = 2 * Y + ((d >> 1) & 1), xx = 2 * X + (d & 1);
+        const bf8 v = load8(x + ((((size_t)z * H + yy) * W + xx) * C8 + c) * 8);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s[k] += v.get(k);
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s[k] *= 0.125f;
+    *reinterpret_cast<uint4 *>(y + 8 * i) = bf8::of(s).q;
 }
 
 // gx[v] += gy[parent(v)] / 8
@@ -463,13 +531,15 @@ cudaError_t nn_weight_flip(const void *w, void *wt, int Cin, int Cout, int Kp, i
 
 cudaError_t nn_elementwise(int op, const void *a, const void *b, void *out, size_t n,
                            cudaStream_t st) {
+    const bool vec = ((uintptr_t)a | (uintptr_t)(op == 1 || op == 3 ? nullptr : b) | (uintptr_t)out) % 16 == 0;
+    const size_t n8 = vec ? n / 8 : 0;
+    const unsigned blocks = nblk(n8 + (n - 8 * n8));
+    const auto *bb = (const __nv_bfloat16 *)b;
+    auto *ob = (__nv_bfloat16 *)out;
     switch (op) {
-        case 0: k_relu_bwd<<<nblk(n), 256, 0, st>>>((const float *)a, (const __nv_bfloat16 *)b,
-                                                    (__nv_bfloat16 *)out, n); break;
-        case 1: k_cast_bf16<<<nblk(n), 256, 0, st>>>((const float *)a, (__nv_bfloat16 *)out, n); break;
-        case 2: k_add_bf16<<<nblk(n), 256, 0, st>>>((const __nv_bfloat16 *)a,
-                                                     (const __nv_bfloat16 *)b,
-                                                     (__nv_bfloat16 *)out, n); break;
+        case 0: k_to_bf16<0><<<blocks, 256, 0, st>>>(a, bb, ob, n8, n); break;
+        case 1: k_to_bf16<1><<<blocks, 256, 0, st>>>(a, bb, ob, n8, n); break;
+        case 2: k_to_bf16<2><<<blocks, 256, 0, st>>>(a, bb, ob, n8, n); break;
         case 3: k_accum_f32<<<nblk(n), 256, 0, st>>>((const float *)a, (float *)out, n); break;
         default: return cudaErrorInvalidValue;
     }
@@ -479,8 +549,14 @@ cudaError_t nn_elementwise(int op, const void *a, const void *b, void *out, size
 cudaError_t nn_resample(int op, const void *x, void *y, int D, int H, int W, int C, cudaStream_t st) {
     // D, H, W: the fine (large) size for pooling ops, the coarse size for upsampling ops
     switch (op) {
-        case 0: k_avgpool2<<<nblk((size_t)D * H * W * C / 8), 256, 0, st>>>(
-                    (const __nv_bfloat16 *)x, (__nv_bfloat16 *)y, D, H, W, C); break;
+        case 0:
+            if (C % 8 == 0 && (uintptr_t)x % 16 == 0 && (uintptr_t)y % 16 == 0)
+                k_avgpool2_v8<<<nblk((size_t)D * H * W * C / 64), 256, 0, st>>>(
+                    (const __nv_bfloat16 *)x, (__nv_bfloat16 *)y, D, H, W, C / 8);
+            else
+                k_avgpool2<<<nblk((size_t)D * H * W * C / 8), 256, 0, st>>>(
+                    (const __nv_bfloat16 *)x, (__nv_bfloat16 *)y, D, H, W, C);
+            break;
         case 1: k_avgpool2_bwd<<<nblk((size_t)D * H * W * C), 256, 0, st>>>(
                     (const float *)x, (float *)y, D, H, W, C); break;
         case 2:

@@ -195,6 +195,7 @@ class UNet3D:
     # -- forward / backward ------------------------------------------------------
     def forward(self, feat, dims, keep=False):
         """feat: BF16 [V][3]; returns FP32 [V][2] (and the activations if keep)."""
+        import torch
         c1, c2, c3, c4 = self.widths
         d1 = dims
         d2 = tuple(n // 2 for n in d1)
@@ -214,15 +215,15 @@ class UNet3D:
         a["b2"] = self.bott[1].forward(a["b1"], d4)
         a["u3"] = upsample(a["b2"], d4, c4)
         a["d3a"] = self.dec3[0].forward(a["u3"], d3)
-        a["a3"] = elementwise(2, a["d3a"], a["s3"], a["d3a"].clone())
+        a["a3"] = elementwise(2, a["d3a"], a["s3"], torch.empty_like(a["d3a"]))
         a["d3"] = self.dec3[1].forward(a["a3"], d3)
         a["u2"] = upsample(a["d3"], d3, c3)
         a["d2a"] = self.dec2[0].forward(a["u2"], d2)
-        a["a2"] = elementwise(2, a["d2a"], a["s2"], a["d2a"].clone())
+        a["a2"] = elementwise(2, a["d2a"], a["s2"], torch.empty_like(a["d2a"]))
         a["d2"] = self.dec2[1].forward(a["a2"], d2)
         a["u1"] = upsample(a["d2"], d2, c2)
         a["d1a"] = self.dec1[0].forward(a["u1"], d1)
-        a["a1"] = elementwise(2, a["d1a"], a["s1"], a["d1a"].clone())
+        a["a1"] = elementwise(2, a["d1a"], a["s1"], torch.empty_like(a["d1a"]))
         a["d1"] = self.dec1[1].forward(a["a1"], d1)
         pred = self.head.forward(a["d1"], d1, out_bf16=False)
         if keep:
