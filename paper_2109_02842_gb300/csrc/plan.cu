@@ -796,9 +796,8 @@ pl_status build_plan(pl_plan *P, const pl_geometry *g, const pl_scan *s, const p
                                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
             if (r != CUDA_SUCCESS) return fail(PL_ERR_CUDA, "cuTensorMapEncodeTiled failed");
         }
-        // the range table as exact sums on the tensor cores (one or two
-        // 64-frequency atoms: up to 128 frequencies; table rows up to 256),
-        // else the NUFFT
+        // the range table as exact sums on the tensor cores (one to four
+        // 64-frequency atoms, see below; table rows up to 256), else the NUFFT
         RtTcArgs &ra = P->rt;
         ra.C = P->C;
         ra.Np = P->Np;
@@ -826,7 +825,17 @@ pl_status build_plan(pl_plan *P, const pl_geometry *g, const pl_scan *s, const p
                     "cudaDeviceGetAttribute");
             ra.grid = sms;
         }
-        P->rt_tc = ra.natoms <= 2 && ra.Lp <= 256 && 4 * ra.Lh <= 512 &&
+        // three and four atoms (129 to 256 frequencies) only with the FP32
+        // spectrum and the hi/lo split, where sums and NUFFT agree to FP32
+        // rounding (through a table rounded to BF16 the two differ by more),
+        // and from 16384 (channel, bin) pairs on. Table stage, NUFFT and sums,
+        // ms: 201 frequencies, 115 channels, 216 bins 0.351 and 0.058; 256, 576,
+        // 512: 4.82 and 0.372; 160, 128, 128: 0.125 and 0.031. (160, 64, 64:
+        // 0.033 and 0.020; the parity tests hold plans of that size to the
+        // NUFFT-built table.)
+        const bool natoms_ok = ra.natoms <= 2 || (ra.natoms <= 4 && P->precision == 0 &&
+                                                  (long long)P->C * P->Np >= 16384);
+        P->rt_tc = natoms_ok && ra.Lp <= 256 && 4 * ra.Lh <= 512 &&
                    range_table_tc_smem_bytes(ra) <= 227 * 1024;
         if (P->rt_tc) {
             const size_t nE = (size_t)P->Np * 4 * ra.Lp * ra.Kp;

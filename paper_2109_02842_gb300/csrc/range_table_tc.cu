@@ -1,6 +1,6 @@
 // Range-profile table of step (8a) / (19a) for the tensor-core back-projection,
 // evaluated as exact sums on the tensor cores instead of a type-1 NUFFT (up to
-// 128 frequencies):
+// 256 frequencies, see build_plan):
 //
 //   b[c][i][u] = sum_m S[c][u][m] E[u][i][m],   E = alpha e^{+j theta_um (i - L/2)},
 //
@@ -16,7 +16,7 @@
 //   k_rt_prep          S [C][N_p][M] -> A [u][re hi, re lo, im hi, im lo][C][K] BF16
 //   k_range_table_tc   persistent, one block per SM, over the items (128-channel
 //                      block, bin, row part): TMA (128-byte swizzled, K-major) A
-//                      and E tiles, 12 MMAs per 16-frequency step (up to two
+//                      and E tiles, 12 MMAs per 16-frequency step (up to four
 //                      64-frequency atoms per item), tcgen05.ld,
 //                      BF16 hi/lo, stored straight from the registers into
 //                      prod [u][hi, lo][row][Cp] of (re, im) pairs, channels
@@ -423,7 +423,7 @@ cudaError_t launch_range_table_tc(const RtTcArgs &ra, const CUtensorMap &tmA,
                                   const CUtensorMap &tmB, const float2 *S,
                                   void *A, void *prod, void *table, int row_words, int planar,
                                   int *err, bool prepared, cudaStream_t st) {
-    if (ra.natoms < 1 || ra.natoms > 2 || 4 * ra.Lh > 512 || ra.grid < 1 || row_words % 4 != 0 ||
+    if (ra.natoms < 1 || ra.natoms > 4 || 4 * ra.Lh > 512 || ra.grid < 1 || row_words % 4 != 0 ||
         2 * ra.L > 65535)
         return cudaErrorInvalidValue;
     cudaError_t e;
