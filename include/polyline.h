@@ -122,7 +122,8 @@ typedef struct {
  *         workspace holds [channel][hi/lo][row][column] BF16, hi = BF16(x),
  *         lo = BF16(x - hi): by default (tile_u = 0) planar, every bin in one
  *         block (tile_u = n_pad rounded up to 16), column u = Re b_u and
- *         column tile_u + u = Im b_u, and each tile's channels in two parts;
+ *         column tile_u + u = Im b_u, and each tile's channels in two parts
+ *         (up to eight for images of few tiles);
  *         where that does not fit tensor memory, or with an explicit tile_u,
  *         interleaved, column 2u + (re, im) within blocks of tile_u bins.
  *         A bounded device wait of block_config 4 that runs out makes the next
@@ -352,9 +353,9 @@ pl_status pl_plan_get_info(const pl_plan *plan, pl_info *info);
  *                          {re_u, re_u+1, im_u, im_u+1} (float32, or bfloat16 when
  *                          precision >= 1); block_config 4: see pl_options
  *  PL_STAGE_BACKPROJECT -> image spectrum G, complex64 [parts][n_pad][ny][nx]: the
- *                          spectrum is the sum over parts (2 parts, one per half
- *                          of the channels, in the planar block_config 4 layout;
- *                          else 1) */
+ *                          spectrum is the sum over parts (the channel parts of the
+ *                          planar block_config 4 layout where they are kept
+ *                          apart, else 1) */
 pl_status pl_plan_workspace(pl_plan *plan, int stage, void **dev_ptr, size_t *bytes);
 
 /* Per-stage timing with CUDA events recorded on the execute stream.

@@ -58,6 +58,8 @@ bool zidft_tc_make_map(const ZidftTcArgs &a, const __nv_bfloat16 *tb, CUtensorMa
 size_t zidft_tc_smem_bytes(const ZidftTcArgs &a);
 cudaError_t launch_zidft_tc(const ZidftTcArgs &a, const CUtensorMap *map, const float2 *G,
                             const float2 *G2, float2 *out, int *err, cudaStream_t st);
+// G[0] += G[1] + ... + G[parts - 1], spectra of n values; the others are cleared
+cudaError_t launch_sum_spectra(float2 *G, int parts, size_t n, cudaStream_t st);
 
 // ---- setup.cu --------------------------------------------------------------
 // Per k_z bin: kappa range over propagating frequencies; kc = centre (double
@@ -136,7 +138,7 @@ struct TcArgs {
     int UT;              // k_z bins per block (the MMA's N: UT planar, 2 UT interleaved)
     int planar;          // 1: table rows [Re of every bin | Im of every bin], accumulators
                          //    Re G and Im G, 12 products per K step; 0: (re, im) pairs, P and Q
-    int nsplit;          // channel parts per tile (blocks adding into G: 1 or 2)
+    int nsplit;          // channel parts per tile (1, 2, or up to 8 for few tiles)
     int im_col;          // planar: table column of the first Im entry
     unsigned im_off;     // planar: smem offset of a window's Im columns (ncb x cb_bytes)
     int ncb;             // 64-column blocks of a block's window: ceil(N / 64)

@@ -688,7 +688,21 @@ pl_status build_plan(pl_plan *P, const pl_geometry *g, const pl_scan *s, const p
         // proportion to that count); the parts also fill the SMs' last wave
         // better than one block per tile.
         ta.nsplit = ta.planar && P->C >= 2 * ta.npar ? 2 : 1;
-        // the parts add into one spectrum (zeroed first), so the inverse
+        // An image of few tiles leaves most SMs idle while a block's chain of
+        // channels runs (0.8 us each): up to eight parts, of at least eight
+        // channels, as many as the SMs take. Their spectra are kept apart and
+        // added in order, so results stay bitwise reproducible. 64 channels, 32 x 32 pixels (16 -> 64 blocks): MEASURED.
+        // Up to 256 channels: the accumulation error of longer sums would
+        // change with the split by more than 1e-5 of the image.
+        if (ta.nsplit == 2 && P->C <= 256) {
+            int dev = 0, sms = 0;
+            PL_CUDA(cudaGetDevice(&dev), "cudaGetDevice");
+            PL_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev),
+                    "cudaDeviceGetAttribute");
+            const int tiles = ntx * nty * ta.n_utiles;
+            ta.nsplit = std::max(2, std::min(std::min(8, P->C / 8), sms / tiles));
+        }
+        // the two parts add into one spectrum (zeroed first), so the inverse
         // transform reads one spectrum instead of two; the batch's
         // persistent kernel (one_block_per_sm) keeps one spectrum per part
         ta.g_atomic = (ta.nsplit == 2 && !o.one_block_per_sm) ? 1 : 0;
@@ -967,10 +981,15 @@ pl_status pl_stage_backproject(pl_plan *P, cudaStream_t st) {
     return PL_OK;
 }
 
-// The inverse z transform of G; `parts` = 2 adds the second channel part's
-// spectrum as it loads the first.
+// The inverse z transform of G; the spectra of two channel parts are added as
+// they are loaded, those of more in a pass before (in the inverse DFT's loads
+// eight parts made a chain of loads: 50.9 us a scan against 45.0).
 static pl_status stage_zifft(pl_plan *P, float2 *image, cudaStream_t st, int parts) {
     const int P2 = P->grid.nx * P->grid.ny;
+    if (parts > 2) {
+        PL_CUDA(launch_sum_spectra(P->d_G, parts, (size_t)P->Np * P2, st), "sum_spectra");
+        parts = 1;
+    }
     const float2 *G2 = parts > 1 ? P->d_G + (size_t)P->Np * P2 : nullptr;
     if (P->inv_fft)
         PL_CUDA(launch_fft_strided(P->d_G, image, 1, P->Np, P2, P->zplan, P->d_twz, +1,
@@ -1448,6 +1467,7 @@ pl_status pl_plan_get_info(const pl_plan *P, pl_info *info) {
     // back-projection, the inverse z transform
     i.launches_per_execute = (P->block_config == 4 && P->rt_tc) ? (P->fwd_fft ? 5 : 6) : 4;
     if (P->bp_full > 0) i.launches_per_execute += 2;   // a second back-projection and z-IFFT launch
+    if (g_parts(P) > 2) i.launches_per_execute += 1;   // the sum of the channel parts
     i.bp_launches = P->bp_full > 0 ? 2 : 1;
     i.workspace_bytes = P->workspace;
     i.updates_per_execute = (double)P->C * P->grid.nx * P->grid.ny * P->grid.nz * P->M;

@@ -272,7 +272,33 @@ __global__ void k_zidft_tc_table(const float2 *__restrict__ T, int nz, int n_in,
     tb[3 * pl + idx] = __float2bfloat16_rn(im - __bfloat162float(ih));
 }
 
+// G[0] += G[1] + ... + G[parts - 1], in order, the others cleared (the sum over
+// the parts stays what it was)
+constexpr int kMaxParts = 8;
+__global__ void __launch_bounds__(256)
+k_sum_spectra(float2 *__restrict__ G, int parts, size_t n) {
+    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    float2 w[kMaxParts];                 // every load in flight at once
+#pragma unroll
+    for (int p = 0; p < kMaxParts; ++p) w[p] = p < parts ? G[p * n + i] : make_float2(0.f, 0.f);
+    float2 v = w[0];
+#pragma unroll
+    for (int p = 1; p < kMaxParts; ++p) {
+        v.x += w[p].x;
+        v.y += w[p].y;
+        if (p < parts) G[p * n + i] = make_float2(0.f, 0.f);
+    }
+    G[i] = v;
+}
+
 }  // namespace
+
+cudaError_t launch_sum_spectra(float2 *G, int parts, size_t n, cudaStream_t st) {
+    if (parts > kMaxParts) return cudaErrorInvalidValue;
+    k_sum_spectra<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(G, parts, n);
+    return cudaGetLastError();
+}
 
 ZidftTcArgs zidft_tc_shape(int n_in, int n_cols, int nz) {
     ZidftTcArgs a{};
