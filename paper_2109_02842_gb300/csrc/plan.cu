@@ -691,7 +691,9 @@ pl_status build_plan(pl_plan *P, const pl_geometry *g, const pl_scan *s, const p
         // An image of few tiles leaves most SMs idle while a block's chain of
         // channels runs (0.8 us each): up to eight parts, of at least eight
         // channels, as many as the SMs take. Their spectra are kept apart and
-        // added in order, so results stay bitwise reproducible. 64 channels, 32 x 32 pixels (16 -> 64 blocks): MEASURED.
+        // added in order, so results stay bitwise reproducible. Whole scan: 64
+        // channels, 32 x 32 pixels (16 -> 64 blocks) 59.4 -> 45.0 us (49.1 with
+        // four parts), 120 channels, 64 x 64 (64 -> 128 blocks) 76 -> 67 us.
         // Up to 256 channels: the accumulation error of longer sums would
         // change with the split by more than 1e-5 of the image.
         if (ta.nsplit == 2 && P->C <= 256) {
