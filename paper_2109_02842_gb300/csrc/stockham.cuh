@@ -93,9 +93,8 @@ __device__ __forceinline__ void small_dft<8>(float2 (&v)[8], int sgn) {
 
 }  // namespace stockham_detail
 
-// NCOL columns (compile time). COL_FAST: consecutive threads take consecutive
-// columns (use when columns are the contiguous axis); otherwise consecutive j.
-template <int R, bool COL_FAST, int NCOL>
+// NCOL columns (compile time), consecutive threads take consecutive rows.
+template <int R, int NCOL>
 __device__ __forceinline__ void stockham_stage(const float2 *src, float2 *dst, const float2 *tw,
                                                int N, int Ns, int sgn, int cs, int ns) {
     const int nr = N / R;
@@ -106,9 +105,7 @@ __device__ __forceinline__ void stockham_stage(const float2 *src, float2 *dst, c
     // instructions instead of an integer division
     const float inv_ns = 1.0f / (float)Ns;
     for (int it = threadIdx.x; it < items; it += blockDim.x) {
-        int j, col;
-        if (COL_FAST) { j = it / NCOL; col = it - j * NCOL; }
-        else { col = it / nr; j = it - col * nr; }
+        const int col = it / nr, j = it - col * nr;
         const int jh = __float2int_rz(((float)j + 0.5f) * inv_ns);
         const int k = j - jh * Ns;
         const float2 *s = src + col * cs;
@@ -130,7 +127,7 @@ __device__ __forceinline__ void stockham_stage(const float2 *src, float2 *dst, c
 
 // Runs every stage of `plan` on NCOL columns; returns the buffer holding the
 // result. Ends with a __syncthreads().
-template <bool COL_FAST, int NCOL>
+template <int NCOL>
 __device__ __forceinline__ float2 *stockham_run(float2 *buf0, float2 *buf1, const float2 *tw,
                                                 const FftPlan &plan, int sgn, int cs, int ns) {
     float2 *src = buf0, *dst = buf1;
@@ -138,11 +135,11 @@ __device__ __forceinline__ float2 *stockham_run(float2 *buf0, float2 *buf1, cons
     const int N = plan.n;
     for (int s = 0; s < plan.n_stages; ++s) {
         const int R = plan.radix[s];
-        if (R == 8) stockham_stage<8, COL_FAST, NCOL>(src, dst, tw, N, Ns, sgn, cs, ns);
-        else if (R == 4) stockham_stage<4, COL_FAST, NCOL>(src, dst, tw, N, Ns, sgn, cs, ns);
-        else if (R == 2) stockham_stage<2, COL_FAST, NCOL>(src, dst, tw, N, Ns, sgn, cs, ns);
-        else if (R == 3) stockham_stage<3, COL_FAST, NCOL>(src, dst, tw, N, Ns, sgn, cs, ns);
-        else stockham_stage<5, COL_FAST, NCOL>(src, dst, tw, N, Ns, sgn, cs, ns);
+        if (R == 8) stockham_stage<8, NCOL>(src, dst, tw, N, Ns, sgn, cs, ns);
+        else if (R == 4) stockham_stage<4, NCOL>(src, dst, tw, N, Ns, sgn, cs, ns);
+        else if (R == 2) stockham_stage<2, NCOL>(src, dst, tw, N, Ns, sgn, cs, ns);
+        else if (R == 3) stockham_stage<3, NCOL>(src, dst, tw, N, Ns, sgn, cs, ns);
+        else stockham_stage<5, NCOL>(src, dst, tw, N, Ns, sgn, cs, ns);
         __syncthreads();
         float2 *t = src; src = dst; dst = t;
         Ns *= R;

@@ -39,10 +39,13 @@ struct SplitOut {
     int hi_only;             // split output: hi planes only (BF16 spectrum)
     int bf16_rows;           // plain output as bfloat16 (re, im) pairs
 };
-// PAIRS (I even): every access moves two adjacent columns (16-byte copies,
-// float4 shared-memory accesses, column pairs through the FFT stages).
+// The FFT stages run on column pairs (float4 shared-memory accesses, a zero
+// column beside an odd last one). VEC (even rows, 16-byte aligned): the copies
+// and the plain output move pairs too, else single columns (8 bytes).
 // SPLIT: the output is the range table's operand (sp.A), else `out`.
-template <bool PAIRS, bool SPLIT>
+// (Odd rows took single columns through every stage before: a scan of 51
+// frequencies 67.0 -> 65.8 us, of 201 235.9 -> 233.8.)
+template <bool VEC, bool SPLIT>
 __global__ void __launch_bounds__(kFftThreads)
 k_fft_strided(const float2 *__restrict__ in, const float2 *__restrict__ in2, float2 *__restrict__ out,
               int n_in, int I, int ld, FftPlan plan, const float2 *__restrict__ tw_g, int sgn,
@@ -54,8 +57,8 @@ k_fft_strided(const float2 *__restrict__ in, const float2 *__restrict__ in2, flo
     float2 *tw = smem + 2 * N * kFftIB;
     const int i0 = blockIdx.x * kFftIB;
     const size_t b = blockIdx.y;
-    constexpr int CW = PAIRS ? 2 : 1;          // columns per access
-    constexpr int NG = kFftIB / CW;            // accesses per row
+    constexpr int CW = VEC ? 2 : 1;            // columns per copy
+    constexpr int NG = kFftIB / CW;            // copies per row
 
     // the whole panel in flight at once: asynchronous copies, zeros for the
     // padding rows and the columns past I. Each thread keeps one column group
@@ -73,7 +76,7 @@ k_fft_strided(const float2 *__restrict__ in, const float2 *__restrict__ in2, flo
         const size_t src_step = (size_t)RPS * ld;
         for (int n = n_first; n < N; n += RPS, src += src_step, dst += RPS * kFftIB) {
             if (col_ok && n < n_in) {
-                if (PAIRS)
+                if (VEC)
                     asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(
                                      (unsigned)__cvta_generic_to_shared(dst)),
                                  "l"(src)
@@ -83,7 +86,7 @@ k_fft_strided(const float2 *__restrict__ in, const float2 *__restrict__ in2, flo
                                      (unsigned)__cvta_generic_to_shared(dst)),
                                  "l"(src)
                                  : "memory");
-            } else if (PAIRS) {
+            } else if (VEC) {
                 *reinterpret_cast<float4 *>(dst) = make_float4(0.f, 0.f, 0.f, 0.f);
             } else {
                 *dst = make_float2(0.f, 0.f);
@@ -93,96 +96,61 @@ k_fft_strided(const float2 *__restrict__ in, const float2 *__restrict__ in2, flo
     asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
     __syncthreads();
 
-    if constexpr (PAIRS) {
-        // the last FFT stage writes the output rows itself: transform index t
-        // goes to output row (t - out_off) mod N when that is below out_rows
-        if constexpr (SPLIT) {
-            const size_t plane = (size_t)sp.batch * sp.Kp;
-            __nv_bfloat16 *A = sp.A + b * sp.Kp + i0;
-            auto emit = [&](int t, int cp, float2 x0, float2 x1) {
-                int r = t - out_off;
-                if (r < 0) r += N;
-                if (r >= out_rows || i0 + 2 * cp >= I) return;
-                const float2 v0 = cscale(x0, scale), v1 = cscale(x1, scale);
-                const __nv_bfloat16 h0 = __float2bfloat16(v0.x), h1 = __float2bfloat16(v1.x);
-                const __nv_bfloat16 g0 = __float2bfloat16(v0.y), g1 = __float2bfloat16(v1.y);
-                __nv_bfloat16 *o = A + (size_t)r * 4 * plane + 2 * cp;
-                *reinterpret_cast<__nv_bfloat162 *>(o) = __halves2bfloat162(h0, h1);
-                *reinterpret_cast<__nv_bfloat162 *>(o + 2 * plane) = __halves2bfloat162(g0, g1);
-                if (sp.hi_only) return;
-                *reinterpret_cast<__nv_bfloat162 *>(o + plane) = __halves2bfloat162(
-                    __float2bfloat16(v0.x - __bfloat162float(h0)),
-                    __float2bfloat16(v1.x - __bfloat162float(h1)));
-                *reinterpret_cast<__nv_bfloat162 *>(o + 3 * plane) = __halves2bfloat162(
-                    __float2bfloat16(v0.y - __bfloat162float(g0)),
-                    __float2bfloat16(v1.y - __bfloat162float(g1)));
-            };
-            stockham_run_pairs_emit<kFftIB>(buf0, buf1, tw, plan, sgn, in2 != nullptr, emit);
-        } else {
-            float2 *o0 = out + b * out_rows * (size_t)ld + i0;
-            __nv_bfloat162 *ob = reinterpret_cast<__nv_bfloat162 *>(out) + b * out_rows * (size_t)ld + i0;
-            auto emit = [&](int t, int cp, float2 x0, float2 x1) {
-                int r = t - out_off;
-                if (r < 0) r += N;
-                if (r >= out_rows || i0 + 2 * cp >= I) return;
-                if (sp.bf16_rows) {
-                    __nv_bfloat162 q[2] = {__floats2bfloat162_rn(scale * x0.x, scale * x0.y),
-                                           __floats2bfloat162_rn(scale * x1.x, scale * x1.y)};
-                    *reinterpret_cast<uint2 *>(ob + (size_t)r * ld + 2 * cp) =
-                        *reinterpret_cast<const uint2 *>(q);
-                    return;
-                }
-                *reinterpret_cast<float4 *>(o0 + (size_t)r * ld + 2 * cp) =
-                    make_float4(scale * x0.x, scale * x0.y, scale * x1.x, scale * x1.y);
-            };
-            stockham_run_pairs_emit<kFftIB>(buf0, buf1, tw, plan, sgn, in2 != nullptr, emit);
-        }
-        return;
-    }
-
-    if (in2) {
-        for (int idx = threadIdx.x; idx < N * kFftIB / 2; idx += kFftThreads) {
-            float4 *a = reinterpret_cast<float4 *>(buf0) + idx;
-            const float4 c = reinterpret_cast<const float4 *>(buf1)[idx];
-            *a = make_float4(a->x + c.x, a->y + c.y, a->z + c.z, a->w + c.w);
-        }
-        __syncthreads();
-    }
-    // single columns (I odd or unaligned buffers)
-    const float2 *src = stockham_run<true, kFftIB>(buf0, buf1, tw, plan, sgn, 1, kFftIB);
-    // out_off < N and r < out_rows <= N: one conditional subtraction wraps
-    if (!col_ok) return;
+    // the last FFT stage writes the output rows itself: transform index t
+    // goes to output row (t - out_off) mod N when that is below out_rows
     if constexpr (SPLIT) {
+        // (the pair's second column may be the operand's first padding column,
+        // which is zero and stays so)
         const size_t plane = (size_t)sp.batch * sp.Kp;
-        __nv_bfloat16 *o = sp.A + (size_t)n_first * 4 * plane + b * sp.Kp + i0 + col;
-        for (int r = n_first; r < out_rows; r += RPS, o += (size_t)RPS * 4 * plane) {
-            int sr = r + out_off;
-            if (sr >= N) sr -= N;
-            const float2 t = cscale(src[sr * kFftIB + col], scale);
-            const __nv_bfloat16 h = __float2bfloat16(t.x), g = __float2bfloat16(t.y);
-            o[0] = h;
-            o[2 * plane] = g;
-            if (!sp.hi_only) {
-                o[plane] = __float2bfloat16(t.x - __bfloat162float(h));
-                o[3 * plane] = __float2bfloat16(t.y - __bfloat162float(g));
-            }
-        }
-    } else if (sp.bf16_rows) {
-        __nv_bfloat162 *o = reinterpret_cast<__nv_bfloat162 *>(out) +
-                            (b * out_rows + n_first) * (size_t)ld + i0 + col;
-        for (int r = n_first; r < out_rows; r += RPS, o += (size_t)RPS * ld) {
-            int sr = r + out_off;
-            if (sr >= N) sr -= N;
-            const float2 t = cscale(src[sr * kFftIB + col], scale);
-            *o = __floats2bfloat162_rn(t.x, t.y);
-        }
+        __nv_bfloat16 *A = sp.A + b * sp.Kp + i0;
+        auto emit = [&](int t, int cp, float2 x0, float2 x1) {
+            int r = t - out_off;
+            if (r < 0) r += N;
+            if (r >= out_rows || i0 + 2 * cp >= I) return;
+            const float2 v0 = cscale(x0, scale), v1 = cscale(x1, scale);
+            const __nv_bfloat16 h0 = __float2bfloat16(v0.x), h1 = __float2bfloat16(v1.x);
+            const __nv_bfloat16 g0 = __float2bfloat16(v0.y), g1 = __float2bfloat16(v1.y);
+            __nv_bfloat16 *o = A + (size_t)r * 4 * plane + 2 * cp;
+            *reinterpret_cast<__nv_bfloat162 *>(o) = __halves2bfloat162(h0, h1);
+            *reinterpret_cast<__nv_bfloat162 *>(o + 2 * plane) = __halves2bfloat162(g0, g1);
+            if (sp.hi_only) return;
+            *reinterpret_cast<__nv_bfloat162 *>(o + plane) = __halves2bfloat162(
+                __float2bfloat16(v0.x - __bfloat162float(h0)),
+                __float2bfloat16(v1.x - __bfloat162float(h1)));
+            *reinterpret_cast<__nv_bfloat162 *>(o + 3 * plane) = __halves2bfloat162(
+                __float2bfloat16(v0.y - __bfloat162float(g0)),
+                __float2bfloat16(v1.y - __bfloat162float(g1)));
+        };
+        stockham_run_pairs_emit<kFftIB>(buf0, buf1, tw, plan, sgn, in2 != nullptr, emit);
     } else {
-        float2 *o = out + (b * out_rows + n_first) * (size_t)ld + i0 + col;
-        for (int r = n_first; r < out_rows; r += RPS, o += (size_t)RPS * ld) {
-            int sr = r + out_off;
-            if (sr >= N) sr -= N;
-            *o = cscale(src[sr * kFftIB + col], scale);
-        }
+        float2 *o0 = out + b * out_rows * (size_t)ld + i0;
+        __nv_bfloat162 *ob = reinterpret_cast<__nv_bfloat162 *>(out) + b * out_rows * (size_t)ld + i0;
+        auto emit = [&](int t, int cp, float2 x0, float2 x1) {
+            int r = t - out_off;
+            if (r < 0) r += N;
+            if (r >= out_rows || i0 + 2 * cp >= I) return;
+            const size_t at = (size_t)r * ld + 2 * cp;
+            const bool both = VEC || i0 + 2 * cp + 1 < I;
+            if (sp.bf16_rows) {
+                __nv_bfloat162 q[2] = {__floats2bfloat162_rn(scale * x0.x, scale * x0.y),
+                                       __floats2bfloat162_rn(scale * x1.x, scale * x1.y)};
+                if (VEC) {
+                    *reinterpret_cast<uint2 *>(ob + at) = *reinterpret_cast<const uint2 *>(q);
+                } else {
+                    ob[at] = q[0];
+                    if (both) ob[at + 1] = q[1];
+                }
+                return;
+            }
+            if (VEC) {
+                *reinterpret_cast<float4 *>(o0 + at) =
+                    make_float4(scale * x0.x, scale * x0.y, scale * x1.x, scale * x1.y);
+            } else {
+                o0[at] = cscale(x0, scale);
+                if (both) o0[at + 1] = cscale(x1, scale);
+            }
+        };
+        stockham_run_pairs_emit<kFftIB>(buf0, buf1, tw, plan, sgn, in2 != nullptr, emit);
     }
 }
 
@@ -255,14 +223,15 @@ cudaError_t launch_fft_strided(const float2 *in, float2 *out, int batch, int n_i
                                void *split_A, int split_Kp, const float2 *in2, int ld,
                                int bf16_out) {
     const size_t smem = fft_strided_smem_bytes(plan.n);
-    // column pairs need 16-byte aligned rows: I even, 16-byte aligned
-    // buffers, and (split output) an even operand row length
+    // copies of column pairs need 16-byte aligned rows: I even, 16-byte aligned
+    // buffers; the split output always takes pairs (operand rows of Kp, a
+    // multiple of 64)
     if (ld <= 0) ld = I;
+    if (split_A && (split_Kp % 2 || (uintptr_t)split_A % 4 || split_Kp < (I + 1) / 2 * 2))
+        return cudaErrorInvalidValue;
     if (ld < I) return cudaErrorInvalidValue;
     const bool pairs = (I % 2 == 0) && (ld % 2 == 0) && ((uintptr_t)in % 16 == 0) &&
-                       ((uintptr_t)in2 % 16 == 0) &&
-                       (split_A ? (split_Kp % 2 == 0 && (uintptr_t)split_A % 4 == 0)
-                                : (uintptr_t)out % 16 == 0);
+                       ((uintptr_t)in2 % 16 == 0) && (split_A || (uintptr_t)out % 16 == 0);
     auto kern = split_A ? (pairs ? k_fft_strided<true, true> : k_fft_strided<false, true>)
                         : (pairs ? k_fft_strided<true, false> : k_fft_strided<false, false>);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
