@@ -133,12 +133,23 @@ __device__ __forceinline__ void channel_taps(const BpDesc &p, const CoefTable &c
     const float pos = (dl + g.off) * p.inv_h;
     o = min(max((int)ceilf(pos - 0.5f * W), 0), ROWS - W);
     const float s = fmaf(2.0f, pos - (float)o, -(float)(W - 1));
+    // the kernel is even: tap W - 1 - t at s is tap t at -s, so a pair of taps
+    // shares the even and the odd part of one polynomial: 24 FMA for six taps
+    // in place of 42. Whole scans, two runs: 1024 pairs, 192 x 192 pixels, 128
+    // bins, BF16 758 -> 740 and 755 us; 384 channels, 256 x 256, 200 bins 815 ->
+    // 795 us. (Not kept: the rotation below by the bits of r, 762 us, and the
+    // channel's phase from a table, 746 where this alone took 740.)
+    const float s2 = s * s;
 #pragma unroll
-    for (int t = 0; t < W; ++t) {
-        float acc = ct.c[t][ND - 1];
+    for (int t = 0; t < W / 2; ++t) {
+        float ev = ct.c[t][ND - 2], od = ct.c[t][ND - 1];
 #pragma unroll
-        for (int d = ND - 2; d >= 0; --d) acc = fmaf(acc, s, ct.c[t][d]);
-        w[t] = acc;
+        for (int d = ND - 4; d >= 0; d -= 2) {
+            ev = fmaf(ev, s2, ct.c[t][d]);
+            od = fmaf(od, s2, ct.c[t][d + 1]);
+        }
+        w[t] = fmaf(s, od, ev);
+        w[W - 1 - t] = fmaf(-s, od, ev);
     }
     // carrier e^{j kappa_T a} = e^{j (kappa_T delta + (kappa_T a* mod 2 pi))}
     const float th = fmaf(kT.x, dl, bp::phase_ff(kT.x, kT.y, g.a_hi, g.a_lo));

@@ -198,12 +198,19 @@ __device__ __forceinline__ void bp_tile(const BpDesc &p, const CoefTable &ct,
                 const int o = min(max(i0[k] - base, 0), PX - 1);
                 const float s = fmaf(2.0f, pos[k] - (float)(base + o), -(float)(W - 1));
                 float w[W];
+                // (tap W - 1 - t at s is tap t at -s: a pair shares the even and
+                // the odd part of one polynomial)
+                const float s2 = s * s;
 #pragma unroll
-                for (int t = 0; t < W; ++t) {
-                    float acc = ct.c[t][ND - 1];
+                for (int t = 0; t < W / 2; ++t) {
+                    float ev = ct.c[t][ND - 2], od = ct.c[t][ND - 1];
 #pragma unroll
-                    for (int d = ND - 2; d >= 0; --d) acc = fmaf(acc, s, ct.c[t][d]);
-                    w[t] = acc;
+                    for (int d = ND - 4; d >= 0; d -= 2) {
+                        ev = fmaf(ev, s2, ct.c[t][d]);
+                        od = fmaf(od, s2, ct.c[t][d + 1]);
+                    }
+                    w[t] = fmaf(s, od, ev);
+                    w[W - 1 - t] = fmaf(-s, od, ev);
                 }
 #pragma unroll
                 for (int t = 0; t < WT; ++t) {
