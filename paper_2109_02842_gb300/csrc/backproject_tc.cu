@@ -139,17 +139,30 @@ __device__ __forceinline__ void channel_taps(const BpDesc &p, const CoefTable &c
     // bins, BF16 758 -> 740 and 755 us; 384 channels, 256 x 256, 200 bins 815 ->
     // 795 us. (Not kept: the rotation below by the bits of r, 762 us, and the
     // channel's phase from a table, 746 where this alone took 740.)
-    const float s2 = s * s;
+    // (Four taps keep one polynomial each: a plan with four taps makes the
+    // learned path's input, whose BF16 roundings carry a change of its last
+    // bits to 3e-4 of the network's image.)
+    if constexpr (W == 4) {
 #pragma unroll
-    for (int t = 0; t < W / 2; ++t) {
-        float ev = ct.c[t][ND - 2], od = ct.c[t][ND - 1];
+        for (int t = 0; t < W; ++t) {
+            float acc = ct.c[t][ND - 1];
 #pragma unroll
-        for (int d = ND - 4; d >= 0; d -= 2) {
-            ev = fmaf(ev, s2, ct.c[t][d]);
-            od = fmaf(od, s2, ct.c[t][d + 1]);
+            for (int d = ND - 2; d >= 0; --d) acc = fmaf(acc, s, ct.c[t][d]);
+            w[t] = acc;
         }
-        w[t] = fmaf(s, od, ev);
-        w[W - 1 - t] = fmaf(-s, od, ev);
+    } else {
+        const float s2 = s * s;
+#pragma unroll
+        for (int t = 0; t < W / 2; ++t) {
+            float ev = ct.c[t][ND - 2], od = ct.c[t][ND - 1];
+#pragma unroll
+            for (int d = ND - 4; d >= 0; d -= 2) {
+                ev = fmaf(ev, s2, ct.c[t][d]);
+                od = fmaf(od, s2, ct.c[t][d + 1]);
+            }
+            w[t] = fmaf(s, od, ev);
+            w[W - 1 - t] = fmaf(-s, od, ev);
+        }
     }
     // carrier e^{j kappa_T a} = e^{j (kappa_T delta + (kappa_T a* mod 2 pi))}
     const float th = fmaf(kT.x, dl, bp::phase_ff(kT.x, kT.y, g.a_hi, g.a_lo));

@@ -695,8 +695,10 @@ pl_status build_plan(pl_plan *P, const pl_geometry *g, const pl_scan *s, const p
         // channels, 32 x 32 pixels (16 -> 64 blocks) 59.4 -> 45.0 us (49.1 with
         // four parts), 120 channels, 64 x 64 (64 -> 128 blocks) 76 -> 67 us.
         // Up to 256 channels: the accumulation error of longer sums would
-        // change with the split by more than 1e-5 of the image.
-        if (ta.nsplit == 2 && P->C <= 256) {
+        // change with the split by more than 1e-5 of the image. Not with four
+        // taps: such a plan makes the learned path's input, whose BF16
+        // roundings carry a change of its last bits to 3e-4 of its image.
+        if (ta.nsplit == 2 && P->C <= 256 && W != 4) {
             int dev = 0, sms = 0;
             PL_CUDA(cudaGetDevice(&dev), "cudaGetDevice");
             PL_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev),
