@@ -111,7 +111,7 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t &hi, uint32_t 
 // (0 <= o <= ROWS - w for a window of ROWS rows), the tap weights and the
 // carrier e^{j kappa_T a} (sin, cos). The pixel sits (ddx, ddy) from the tile
 // centre; g holds the channel's geometry relative to that centre.
-template <int W, int ROWS>
+template <int W, int ROWS, int SPLIT>
 __device__ __forceinline__ void channel_taps(const BpDesc &p, const CoefTable &ct, const TileGeo &g,
                                              float ddx, float ddy, float2 kT, int &o,
                                              float (&w)[W], float &sn, float &cs) {
@@ -135,14 +135,13 @@ __device__ __forceinline__ void channel_taps(const BpDesc &p, const CoefTable &c
     const float s = fmaf(2.0f, pos - (float)o, -(float)(W - 1));
     // the kernel is even: tap W - 1 - t at s is tap t at -s, so a pair of taps
     // shares the even and the odd part of one polynomial: 24 FMA for six taps
-    // in place of 42. Whole scans, two runs: 1024 pairs, 192 x 192 pixels, 128
-    // bins, BF16 758 -> 740 and 755 us; 384 channels, 256 x 256, 200 bins 815 ->
-    // 795 us. (Not kept: the rotation below by the bits of r, 762 us, and the
-    // channel's phase from a table, 746 where this alone took 740.)
-    // (Four taps keep one polynomial each: a plan with four taps makes the
-    // learned path's input, whose BF16 roundings carry a change of its last
-    // bits to 3e-4 of the network's image.)
-    if constexpr (W == 4) {
+    // in place of 42 (384 channels, 256 x 256 pixels, 200 bins: 812 -> 798 us a
+    // scan). Not where a last bit of the weights can flip a BF16 rounding:
+    // BF16-only products (single voxels move by 1e-3 of the image), and four
+    // taps (such a plan makes the learned path's BF16 input, whose roundings
+    // its network carries to 3e-4 of its image). (Not kept: the rotation below
+    // by the bits of r, and the channel's phase from a table: both slower.)
+    if constexpr (W == 4 || SPLIT != 3) {
 #pragma unroll
         for (int t = 0; t < W; ++t) {
             float acc = ct.c[t][ND - 1];
@@ -241,7 +240,7 @@ __device__ __forceinline__ void bp_tc_item(const BpDesc &p, const CoefTable &ct,
             if (cnext < ce) gn = tg[cnext];
             int o;
             float w[W], sn, cs;
-            channel_taps<W, 16 * KS>(p, ct, g, ddx, ddy, kT, o, w, sn, cs);
+            channel_taps<W, 16 * KS, SPLIT>(p, ct, g, ddx, ddy, kT, o, w, sn, cs);
             // element o of the row starts word o / 2; an odd o puts a zero first
             const bool odd = (o & 1) != 0;
             float e[W + 2];
@@ -782,7 +781,7 @@ __device__ __forceinline__ void bp_tc_item_sp(const BpDesc &p, const CoefTable &
             if (c + STEP < ce) gn = tg[c + STEP];
             int o;
             float w[W], sn, cs;
-            channel_taps<W, RW>(p, ct, g, ddx, ddy, kT, o, w, sn, cs);
+            channel_taps<W, RW, SPLIT>(p, ct, g, ddx, ddy, kT, o, w, sn, cs);
             // planar: a1 = [Re A | -Im A], a3 = [Im A | Re A] over [Re rows |
             // Im rows]; interleaved (32 rows): a1 = Re A, a3 = Im A
             uint32_t a1h[8], a3h[8], a1l[8], a3l[8], mA, mB;
