@@ -1,8 +1,9 @@
 // The learned path's 3 x 3 x 3 convolution on the fifth-generation tensor
-// cores (tcgen05), for the shapes the network runs at full size: Cin a
-// multiple of 16, Cout in 1..16 (the MMA's N = 16) or {32, 64, 128}, rows of W
-// in {16, 32, 64, 128} voxels with 128 / W dividing H. Other shapes (the
-// 3-channel input layer, odd sizes) keep the mma.sync kernel of nn.cu.
+// cores (tcgen05): Cin a multiple of 16, Cout in 1..16 (the MMA's N = 16) or
+// {32, 64, 128}, rows of W in {16, 32, 64, 128} voxels with 128 / W dividing H.
+// It takes the wide layers of many tiles and those nn_conv_mma.cu has no room
+// for (the rule and its figures are in nn.cu); narrow layers, other rows and
+// one to four input channels are faster in nn_conv_mma.cu and nn_conv_small.cu.
 //
 // Implicit GEMM: out[v][co] = act(bias[co] + sum_{tap, ci} x[v + off(tap)][ci]
 // w[co][tap Cin + ci]). A tile is 128 consecutive voxels (the MMA's M: 128 / W
