@@ -58,44 +58,52 @@ __device__ __forceinline__ ff ff_dist2d(ff x, ff y, ff px, ff py) {
     return ff_sqrt(ff_add(ff_sqr(dx), ff_sqr(dy)));
 }
 
-// G[u][pixel] of the exact sum: UT bins x a tile of 16 x 8 pixels per block,
-// one pixel per thread.
+// G[u][pixel] of the exact sum: two bins x 128 consecutive pixels per block, one
+// pixel per thread.
 //
 // Bound by the two MUFU operations of a term (16 lanes per cycle and SM). The
-// phase kappa a is split at the tile's reference pixel, a = a_ref + delta:
-// e^{j kappa a_ref} is common to the block and goes into the term's
-// coefficient (k_m S e^{j kappa a_ref}, formed once per block and staged in
-// shared memory, the phase as a float pair), so a (pixel, term) costs one
-// product kappa delta, a sine and a cosine and four FMA in place of a
-// float-float product with its reduction. The launcher keeps kappa delta
-// below kMaxSplitPhase, where a rounded FP32 phase is off by at most 1e-5 rad
-// and by 1e-6 rad on usual grids, independently from term to term.
-// 120 channels, 51 frequencies, 128 bins, 64 x 64 pixels: 4.85 -> 1.65 ms
-// (MUFU floor 1.4 ms). Two bins a block: 1.72 ms with four (512 blocks on 152
-// SMs leave a part-filled last wave), 2.00 ms with eight.
-constexpr int kExTX = 16, kExTY = 8, kExThreads = kExTX * kExTY;
+// terms' coefficients k_m S and wavenumbers are staged in shared memory once per
+// block and read by every lane at once. The phase kappa a of each (pixel, term)
+// is a float-pair product reduced modulo 2 pi, so that the fast sine and cosine
+// see [-pi, pi], where their error is bounded; the two bins' phases are formed
+// in packed pairs. 120 channels, 51 frequencies, 128 bins, 64 x 64 pixels: 4.85
+// (eight bins a block, terms loaded one by one) -> 1.87 ms, 2.29 with unpacked
+// phases (MUFU floor 1.39); 1024 x 1 pixels 4.38 -> 0.62 ms. (Splitting the
+// phase at a reference pixel, one FP32 product of up to 128 rad a term, took
+// 1.65 ms but raised the image's error from 4.7e-6 to 6.4e-6.)
+constexpr int kExThreads = 128;
 constexpr int kExChunk = 256;                 // frequencies staged at a time
-constexpr float kMaxSplitPhase = 128.f;
 
-template <int UT, int MODE>
+// bp::phase_ff of two terms at once in packed pairs (same operations, same
+// rounding), the nearest integer by adding and taking off 1.5 2^23
+__device__ __forceinline__ float2 phase_ff2(float2 kh, float2 kl, float ah, float al) {
+    const float2 h = bp::f2(ah, ah), nh = bp::f2(-ah, -ah);
+    const float2 np = __fmul2_rn(kh, nh);                      // -p
+    float2 e = __ffma2_rn(kh, h, np);
+    e = __ffma2_rn(kh, bp::f2(al, al), e);
+    e = __ffma2_rn(kl, h, e);
+    constexpr float kMagic = 12582912.f;
+    const float2 t = __ffma2_rn(np, bp::f2(-bp::kInvTwoPi, -bp::kInvTwoPi), bp::f2(kMagic, kMagic));
+    const float2 n = __fadd2_rn(t, bp::f2(-kMagic, -kMagic));
+    float2 r = __ffma2_rn(n, bp::f2(bp::kTwoPiHi, bp::kTwoPiHi), np);
+    r = __ffma2_rn(n, bp::f2(bp::kTwoPiLo, bp::kTwoPiLo), r);
+    return __ffma2_rn(r, bp::f2(-1.f, -1.f), e);
+}
+
+template <int MODE>
 __global__ void __launch_bounds__(kExThreads)
 k_exact_sum(ExactDesc e, const float2 *__restrict__ S, const float2 *__restrict__ kap,
             const float *__restrict__ wum, const float4 *__restrict__ chff, float2 *__restrict__ G) {
     // two buffers: one barrier between the staging and the reading of a chunk
     extern __shared__ float4 sm_terms[];
-    __shared__ float2 s_ref[2];
-    const int tiles_x = (e.nx + kExTX - 1) / kExTX;
-    const int ix = (blockIdx.x % tiles_x) * kExTX + (int)threadIdx.x % kExTX;
-    const int iy = (blockIdx.x / tiles_x) * kExTY + (int)threadIdx.x / kExTX;
-    const bool live = ix < e.nx && iy < e.ny;
-    const int u0 = blockIdx.y * UT;
-    // pixels past the edge repeat the last one
-    const ff px = ff_of(e.x0 + min(ix, e.nx - 1) * e.dx), py = ff_of(e.y0 + min(iy, e.ny - 1) * e.dy);
-    const int ref = kExThreads / 2 + kExTX / 2;
+    const int np = e.nx * e.ny, tiles = (np + kExThreads - 1) / kExThreads;
+    const int p = (int)(blockIdx.x % tiles) * kExThreads + (int)threadIdx.x;
+    const int u0 = (int)(blockIdx.x / tiles) * 2;
+    const bool live = p < np;
+    const int ix = live ? p % e.nx : 0, iy = live ? p / e.nx : 0;
+    const ff px = ff_of(e.x0 + ix * e.dx), py = ff_of(e.y0 + iy * e.dy);
     const int mc_full = min(e.n_f, kExChunk);
-    float2 acc[UT];
-#pragma unroll
-    for (int j = 0; j < UT; ++j) acc[j] = make_float2(0.f, 0.f);
+    float2 acc0 = make_float2(0.f, 0.f), acc1 = acc0;
     int buf = 0;
     for (int c = 0; c < e.n_chan; ++c) {
         const float4 t = chff[2 * c], r = chff[2 * c + 1];
@@ -103,101 +111,48 @@ k_exact_sum(ExactDesc e, const float2 *__restrict__ S, const float2 *__restrict_
         // rho_T + rho_R (multi: kappa = sqrt(k^2 - k_z^2 / 4))
         ff a = ff_dist2d(px, py, {t.x, t.y}, {t.z, t.w});
         if (MODE == 1) a = ff_add(a, ff_dist2d(px, py, {r.x, r.y}, {r.z, r.w}));
-        // (two slots: the slot of channel c is read before channel c + 1's
-        // first barrier, and written again after it)
-        if (threadIdx.x == ref) s_ref[c & 1] = make_float2(a.hi, a.lo);
-        __syncthreads();
-        const float2 ar = s_ref[c & 1];
-        const float delta = (a.hi - ar.x) + (a.lo - ar.y);
         for (int m0 = 0; m0 < e.n_f; m0 += kExChunk) {
             const int mc = min(kExChunk, e.n_f - m0);
-            float4 *terms = sm_terms + (size_t)buf * UT * mc_full;
-            for (int i = threadIdx.x; i < UT * mc; i += kExThreads) {
-                const int j = i / mc, m = m0 + i - j * mc, u = u0 + j;
-                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);     // evanescent, or past the bins
+            // [term][coefficients of both bins (re, re, im, im), wavenumbers
+            // (high, high, low, low)]
+            float *terms = reinterpret_cast<float *>(sm_terms + (size_t)buf * 2 * mc_full);
+            for (int i = threadIdx.x; i < 2 * mc; i += kExThreads) {
+                const int j = i >= mc ? 1 : 0, ml = i - j * mc, m = m0 + ml, u = u0 + j;
+                float2 s = make_float2(0.f, 0.f), k = s;        // evanescent, or past the bins
                 if (u < e.n_pad) {
                     const float w = wum[(size_t)u * e.n_f + m];
                     if (w != 0.f) {
-                        const float2 k = kap[(size_t)u * e.n_f + m];
-                        const float2 s = S[((size_t)c * e.n_pad + u) * e.n_f + m];
-                        float sn, cs;
-                        sincosf(bp::phase_ff(k.x, k.y, ar.x, ar.y), &sn, &cs);
-                        const float sr = s.x * w, si = s.y * w;
-                        v = make_float4(fmaf(sr, cs, -si * sn), fmaf(sr, sn, si * cs), k.x, 0.f);
+                        k = kap[(size_t)u * e.n_f + m];
+                        s = S[((size_t)c * e.n_pad + u) * e.n_f + m];
+                        s = make_float2(s.x * w, s.y * w);
                     }
                 }
-                terms[i] = v;
+                float *o = terms + 8 * ml + j;
+                o[0] = s.x;
+                o[2] = s.y;
+                o[4] = k.x;
+                o[6] = k.y;
             }
             __syncthreads();
-#pragma unroll
-            for (int j = 0; j < UT; ++j) {
-                const float4 *tj = terms + j * mc;
-                float2 s = acc[j];
+            const float4 *tm = reinterpret_cast<const float4 *>(terms);
 #pragma unroll 4
-                for (int m = 0; m < mc; ++m) {
-                    const float4 v = tj[m];
-                    float sn, cs;
-                    __sincosf(v.z * delta, &sn, &cs);
-                    s.x = fmaf(v.x, cs, fmaf(-v.y, sn, s.x));
-                    s.y = fmaf(v.x, sn, fmaf(v.y, cs, s.y));
-                }
-                acc[j] = s;
+            for (int m = 0; m < mc; ++m) {
+                const float4 s = tm[2 * m], k = tm[2 * m + 1];
+                float sn0, cs0, sn1, cs1;
+                const float2 ph = phase_ff2(bp::f2(k.x, k.y), bp::f2(k.z, k.w), a.hi, a.lo);
+                __sincosf(ph.x, &sn0, &cs0);
+                __sincosf(ph.y, &sn1, &cs1);
+                acc0.x = fmaf(s.x, cs0, fmaf(-s.z, sn0, acc0.x));
+                acc0.y = fmaf(s.x, sn0, fmaf(s.z, cs0, acc0.y));
+                acc1.x = fmaf(s.y, cs1, fmaf(-s.w, sn1, acc1.x));
+                acc1.y = fmaf(s.y, sn1, fmaf(s.w, cs1, acc1.y));
             }
             buf ^= 1;
         }
     }
     if (live) {
-        const size_t np = (size_t)e.nx * e.ny, p = (size_t)iy * e.nx + ix;
-#pragma unroll
-        for (int j = 0; j < UT; ++j)
-            if (u0 + j < e.n_pad) G[(size_t)(u0 + j) * np + p] = acc[j];
-    }
-}
-
-// The same with the whole phase as a float pair in every term, for pixels so
-// far apart that kappa delta would pass kMaxSplitPhase.
-template <int UT>
-__global__ void __launch_bounds__(128)
-k_exact_sum_coarse(ExactDesc e, const float2 *__restrict__ S, const float2 *__restrict__ kap,
-                   const float *__restrict__ wum, const float4 *__restrict__ chff,
-                   float2 *__restrict__ G) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    const int u0 = blockIdx.y * UT;
-    const int np = e.nx * e.ny;
-    const bool live = p < np;
-    const int ix = live ? p % e.nx : 0, iy = live ? p / e.nx : 0;
-    const ff px = ff_of(e.x0 + ix * e.dx), py = ff_of(e.y0 + iy * e.dy);
-    float2 acc[UT];
-#pragma unroll
-    for (int j = 0; j < UT; ++j) acc[j] = make_float2(0.f, 0.f);
-    for (int c = 0; c < e.n_chan; ++c) {
-        const float4 t = chff[2 * c], r = chff[2 * c + 1];
-        ff a = ff_dist2d(px, py, {t.x, t.y}, {t.z, t.w});
-        if (e.mode == 1) a = ff_add(a, ff_dist2d(px, py, {r.x, r.y}, {r.z, r.w}));
-#pragma unroll
-        for (int j = 0; j < UT; ++j) {
-            const int u = u0 + j;
-            if (u >= e.n_pad) break;
-            const float2 *Su = S + ((size_t)c * e.n_pad + u) * e.n_f;
-            const float2 *ku = kap + (size_t)u * e.n_f;
-            const float *wu = wum + (size_t)u * e.n_f;
-            for (int m = 0; m < e.n_f; ++m) {
-                const float w = wu[m];
-                if (w == 0.f) continue;              // evanescent (uniform across the block)
-                const float2 k = ku[m];
-                const float2 s = Su[m];
-                float sn, cs;
-                __sincosf(bp::phase_ff(k.x, k.y, a.hi, a.lo), &sn, &cs);
-                const float sr = s.x * w, si = s.y * w;
-                acc[j].x = fmaf(sr, cs, fmaf(-si, sn, acc[j].x));
-                acc[j].y = fmaf(sr, sn, fmaf(si, cs, acc[j].y));
-            }
-        }
-    }
-    if (live) {
-#pragma unroll
-        for (int j = 0; j < UT; ++j)
-            if (u0 + j < e.n_pad) G[(size_t)(u0 + j) * np + p] = acc[j];
+        G[(size_t)u0 * np + p] = acc0;
+        if (u0 + 1 < e.n_pad) G[(size_t)(u0 + 1) * np + p] = acc1;
     }
 }
 
@@ -390,31 +345,17 @@ k_bp_direct(DirectDesc e, const float2 *__restrict__ s, const float4 *__restrict
     if (live) img[v] = acc;
 }
 
-template <int UT>
-cudaError_t launch_exact_split(const ExactDesc &e, const float2 *S, const float2 *kap,
-                               const float *wum, const float4 *chff, float2 *G, cudaStream_t st) {
-    const size_t smem = 2 * (size_t)UT * (e.n_f < kExChunk ? e.n_f : kExChunk) * sizeof(float4);
-    const int tiles = ((e.nx + kExTX - 1) / kExTX) * ((e.ny + kExTY - 1) / kExTY);
-    dim3 grid(tiles, (e.n_pad + UT - 1) / UT);
-    if (e.mode == 1) k_exact_sum<UT, 1><<<grid, kExThreads, smem, st>>>(e, S, kap, wum, chff, G);
-    else k_exact_sum<UT, 0><<<grid, kExThreads, smem, st>>>(e, S, kap, wum, chff, G);
-    return cudaGetLastError();
-}
-
 }  // namespace
 
 cudaError_t launch_exact_sum(const ExactDesc &e, const float2 *S, const float2 *kap,
                              const float *wum, const float4 *chff, float2 *G, cudaStream_t st) {
-    // |delta| is at most the distance to the tile's reference pixel (8 and 4
-    // steps away), once per range; kappa <= 2 k (mono) or k per range (multi)
-    const double far = (e.mode == 1 ? 2.0 : 1.0) * hypot(kExTX / 2 * e.dx, kExTY / 2 * e.dy);
-    if (far * e.kappa_max > kMaxSplitPhase) {
-        constexpr int UT = 8;
-        dim3 grid((e.nx * e.ny + 127) / 128, (e.n_pad + UT - 1) / UT);
-        k_exact_sum_coarse<UT><<<grid, 128, 0, st>>>(e, S, kap, wum, chff, G);
-        return cudaGetLastError();
-    }
-    return launch_exact_split<2>(e, S, kap, wum, chff, G, st);
+    // two buffers of 32 bytes a term
+    const size_t smem = 2 * 32 * (size_t)(e.n_f < kExChunk ? e.n_f : kExChunk);
+    const size_t blocks = (size_t)((e.nx * e.ny + kExThreads - 1) / kExThreads) * ((e.n_pad + 1) / 2);
+    if (blocks > 0x7fffffffu) return cudaErrorInvalidValue;
+    auto kern = e.mode == 1 ? k_exact_sum<1> : k_exact_sum<0>;
+    kern<<<(unsigned)blocks, kExThreads, smem, st>>>(e, S, kap, wum, chff, G);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_bp_direct(const DirectDesc &e, const float2 *s, const float4 *chff,

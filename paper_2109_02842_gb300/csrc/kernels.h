@@ -239,7 +239,6 @@ cudaError_t launch_range_table_tc(const RtTcArgs &ra, const CUtensorMap &tmA,
 struct ExactDesc {
     int mode, n_chan, n_pad, n_f, nx, ny;
     double x0, dx, y0, dy;
-    double kappa_max;               // 2 k (mono) or k (multi) of the highest frequency
 };
 struct DirectDesc {
     int mode, n_chan, n_scan, n_f, nx, ny, nz;

@@ -1169,7 +1169,6 @@ static pl_status prepare_comparison(pl_plan *P) {
     e.dx = P->grid.dx;
     e.y0 = P->grid.y0;
     e.dy = P->grid.dy;
-    e.kappa_max = (P->mode == 0 ? 2.0 : 1.0) * P->h_k[P->M - 1];
     DirectDesc &d = P->direct;
     d.mode = P->mode;
     d.n_chan = P->C;
