@@ -39,6 +39,7 @@
 namespace {
 
 constexpr int kWarps = 8, kThreads = 32 * kWarps;
+constexpr int kMaxSmem = 224 * 1024;
 
 struct MmaShape {
     int D, H, W, Cin, Cout, Kp;
@@ -87,7 +88,7 @@ bool conv_mma_plan(int D, int H, int W, int Cin, int Cout, int Kp, MmaShape &bes
                 const int groups = (ty * P + 16 * MT - 1) / (16 * MT);
                 s.xrows = groups * 16 * MT + 2 * P + 2;
                 const size_t smem = mma_smem(s);
-                if (smem > 224 * 1024) break;
+                if (smem > (size_t)kMaxSmem) break;
                 const int occ = smem <= 112 * 1024 ? 2 : 1;
                 const int rounds = (groups + kWarps - 1) / kWarps;
                 // share of the warps' positions that are outputs, times the
@@ -348,7 +349,9 @@ cudaError_t launch_nt(const MmaShape &s, const __nv_bfloat16 *x, const __nv_bflo
                       const float *bias, void *out, int out_bf16, cudaStream_t st) {
     auto kern = out_bf16 ? k_conv3d_mma<NT, MT, true> : k_conv3d_mma<NT, MT, false>;
     const size_t smem = mma_smem(s);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (the same limit whatever the shape: with this call's size, a thread with a
+    // smaller shape could lower it between another thread's call and launch)
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
     if (e != cudaSuccess) return e;
     kern<<<dim3(s.nx * s.ny * s.nz, s.n_co), kThreads, smem, st>>>(x, w, bias, out, s);
     return cudaGetLastError();

@@ -51,6 +51,8 @@ __host__ __device__ constexpr int g_pitch(int MT) { return 16 * MT + 8; }
 
 int mt_of(int Cout) { return Cout <= 16 ? 1 : Cout <= 32 ? 2 : 4; }
 int nt_of(int Cin) { return Cin <= 8 ? 1 : 2; }
+// shared memory a block may take: two blocks an SM up to 32 output channels
+__host__ __device__ constexpr int max_smem(int MT) { return (MT <= 2 ? 112 : 200) * 1024; }
 
 size_t smem_bytes(const WgShape &s) {
     return 2 * (4 * (size_t)s.xrows * x_pitch(nt_of(s.Cin)) +
@@ -70,7 +72,6 @@ WgShape wg_shape(int D, int H, int W, int Cin, int Cout, int Kp) {
     s.Cout = Cout;
     s.Kp = Kp;
     const int MT = mt_of(Cout), NT = nt_of(Cin);
-    const size_t most = (MT <= 2 ? 112 : 200) * 1024;
     s.nx = (W + 63) / 64;
     s.TX = (W + s.nx - 1) / s.nx;
     const int P = s.TX + 2;
@@ -80,7 +81,7 @@ WgShape wg_shape(int D, int H, int W, int Cin, int Cout, int Kp) {
         s.TY = (H + s.ny - 1) / s.ny;
         s.xrows = (s.TY + 2) * P + kSlack;
         s.grows = (s.TY * P + 15) / 16 * 16;
-        if (smem_bytes(s) <= most || ty == 1) break;
+        if (smem_bytes(s) <= (size_t)max_smem(MT) || ty == 1) break;   // (one row: 64 KB at most)
     }
     s.inv_p = ((1u << 20) + P - 1) / P;
     s.n_ci = (Cin + 8 * NT - 1) / (8 * NT);
@@ -311,7 +312,9 @@ cudaError_t launch_one(const WgShape &s, const __nv_bfloat16 *x, const __nv_bflo
                        float *bpart, cudaStream_t st) {
     auto kern = k_wgrad<NT, MT, XVEC, GVEC>;
     const size_t smem = smem_bytes(s);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (the same limit whatever the shape: with this call's size, a thread with a
+    // smaller shape could lower it between another thread's call and launch)
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem(MT));
     if (e != cudaSuccess) return e;
     kern<<<dim3(s.nx * s.ny * s.nz, s.n_ci, s.n_co), kThreads, smem, st>>>(x, gy, part, bpart, s);
     return cudaGetLastError();
