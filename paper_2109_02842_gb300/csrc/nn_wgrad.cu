@@ -52,7 +52,8 @@ __host__ __device__ constexpr int g_pitch(int MT) { return 16 * MT + 8; }
 int mt_of(int Cout) { return Cout <= 16 ? 1 : Cout <= 32 ? 2 : 4; }
 int nt_of(int Cin) { return Cin <= 8 ? 1 : 2; }
 // shared memory a block may take: two blocks an SM up to 32 output channels
-__host__ __device__ constexpr int max_smem(int MT) { return (MT <= 2 ? 112 : 200) * 1024; }
+// (beside the static sb and the 1 KB the system reserves for each)
+__host__ __device__ constexpr int max_smem(int MT) { return (MT <= 2 ? 111 : 200) * 1024; }
 
 size_t smem_bytes(const WgShape &s) {
     return 2 * (4 * (size_t)s.xrows * x_pitch(nt_of(s.Cin)) +
@@ -135,6 +136,23 @@ __device__ __forceinline__ void mma16816(float (&d)[4], const unsigned (&a)[4], 
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+// Running sums: FP32, and a float pair (Knuth's two-sum), rounded once at the end
+struct Plain {
+    float s = 0.f;
+    __device__ __forceinline__ void operator+=(float x) { s += x; }
+    __device__ __forceinline__ float value() const { return s; }
+};
+struct Pair {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void operator+=(float x) {
+        const float s = hi + x, b = s - hi;
+        lo += (hi - (s - b)) + (x - b);
+        hi = s;
+    }
+    // (an infinite sum has no low part: it would be NaN)
+    __device__ __forceinline__ float value() const { return isinf(hi) ? hi : hi + lo; }
+};
+
 // Copies a slice's voxel rows [rows x P] of `C` channels, channels c0 .. c0 +
 // CW, into `dst` (pitch elements per voxel): voxel (y0 + r, x0 + c) of slice z,
 // zeros outside the volume, past column `cols`, and past channel C. VEC: 16
@@ -165,6 +183,7 @@ k_wgrad(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__restrict__ g
         float *__restrict__ part, float *__restrict__ bpart, WgShape s) {
     constexpr int XP = x_pitch(NT), GP = g_pitch(MT);
     extern __shared__ __align__(16) __nv_bfloat16 sm[];
+    __shared__ float sb[kWarps][16 * MT];                  // the warps' bias sums
     __nv_bfloat16 *xs = sm;                                // [4][xrows][XP]
     __nv_bfloat16 *gs = sm + 4 * (size_t)s.xrows * XP;     // [2][grows][GP]
     const int P = s.TX + 2;
@@ -175,7 +194,7 @@ k_wgrad(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__restrict__ g
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, t = lane & 3;
     const int dz = warp / 3, dy = warp % 3;
-    const bool with_bias = bpart != nullptr && blockIdx.y == 0 && warp == 4;
+    const bool with_bias = bpart != nullptr && blockIdx.y == 0;
 
     // the voxels past the slices, and gy's past its rows, stay zero
     for (int i = threadIdx.x; i < 4 * kSlack * XP; i += kThreads) {
@@ -200,7 +219,10 @@ k_wgrad(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__restrict__ g
     };
 
     float acc[3][MT][NT][4] = {};
-    float bacc[MT][4] = {};
+    // bias sums of output channels g and g + 8, over this lane's voxels of this
+    // warp's steps: FP32 additions (products with ones on the tensor cores, which
+    // truncate, were twice as far off for a gradient of one sign)
+    float bacc[MT][2] = {};
 
     // writes partial sum f of the segment and clears the accumulators
     auto store_part = [&](int f) {
@@ -222,11 +244,23 @@ k_wgrad(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__restrict__ g
                             acc[k][i][j][2 * h + q] = 0.f;
                         }
                 if (with_bias) {
-                    if (t == 0 && co < s.Cout) bpart[pi * s.Cout + co] = bacc[i][2 * h];
-                    bacc[i][2 * h] = bacc[i][2 * h + 1] = 0.f;
+                    float b = bacc[i][h];
+                    b += __shfl_xor_sync(0xffffffffu, b, 1);
+                    b += __shfl_xor_sync(0xffffffffu, b, 2);
+                    if (t == 0) sb[warp][i * 16 + g + 8 * h] = b;
+                    bacc[i][h] = 0.f;
                 }
             }
         }
+        if (!with_bias) return;        // (one answer for the whole block)
+        __syncthreads();
+        const int c = (int)threadIdx.x, co = co0 + c;
+        if (c < 16 * MT && co < s.Cout) {
+            Pair b;
+            for (int k = 0; k < kWarps; ++k) b += sb[k][c];
+            bpart[pi * s.Cout + co] = b.value();
+        }
+        __syncthreads();
     };
 
     load_x(z0 - 1);
@@ -249,6 +283,7 @@ k_wgrad(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__restrict__ g
                                      bcol);
         const unsigned ga = smem_u32(gs + ((size_t)(z & 1) * s.grows + arow) * GP + acol);
         const int steps = s.grows / 16;
+        int bst = with_bias ? warp : steps;       // this warp's next step of the bias sum
 #pragma unroll 2
         for (int st = 0; st < steps; ++st) {
             unsigned a[MT][4];
@@ -265,10 +300,15 @@ k_wgrad(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__restrict__ g
 #pragma unroll
                     for (int i = 0; i < MT; ++i) mma16816(acc[k][i][j], a[i], b[2 * j], b[2 * j + 1]);
             }
-            if (with_bias) {
-                constexpr unsigned one2 = 0x3F803F80u;      // (1, 1) in BF16
+            if (st == bst) {
+                bst += kWarps;
+                auto lo = [](unsigned v) { return __uint_as_float(v << 16); };
+                auto hi = [](unsigned v) { return __uint_as_float(v & 0xffff0000u); };
 #pragma unroll
-                for (int i = 0; i < MT; ++i) mma16816(bacc[i], a[i], one2, one2);
+                for (int i = 0; i < MT; ++i)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        bacc[i][h] += (lo(a[i][h]) + hi(a[i][h])) + (lo(a[i][h + 2]) + hi(a[i][h + 2]));
             }
         }
         if ((z + 1 - z0) % s.zsum == 0 || z + 1 == z1) store_part((z - z0) / s.zsum);
@@ -279,31 +319,39 @@ k_wgrad(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__restrict__ g
 
 // gw[co][k] += sum over the parts (k < K), gb[co] += sum over the bias parts:
 // 32 sums a block, kSumWays threads each (every kSumWays-th part, then in order;
-// eight threads with four loads in flight took 0.023 ms for 768 parts)
+// eight threads with four loads in flight took 0.023 ms for 768 parts).
 constexpr int kSumWays = 16;
+template <class T>
+__device__ __forceinline__ void sum_parts(const float *__restrict__ p, float *__restrict__ o,
+                                          float (&s)[kSumWays][32], int nparts, size_t stride,
+                                          bool live) {
+    const int e = threadIdx.x & 31, q = threadIdx.x >> 5;
+    T v;
+    if (live) {
+#pragma unroll 16
+        for (int c = q; c < nparts; c += kSumWays) v += p[(size_t)c * stride];
+    }
+    s[q][e] = v.value();
+    __syncthreads();
+    if (q == 0 && live) {
+        T r;
+        for (int k = 0; k < kSumWays; ++k) r += s[k][e];
+        r += *o;
+        *o = r.value();
+    }
+}
 __global__ void __launch_bounds__(32 * kSumWays)
 k_wgrad_sum(const float *__restrict__ part, const float *__restrict__ bpart, float *__restrict__ gw,
             float *__restrict__ gb, int nparts, int Cout, int K, int Kp, int wblocks) {
     __shared__ float s[kSumWays][32];
-    const int e = threadIdx.x & 31, q = threadIdx.x >> 5;
-    const bool bias = (int)blockIdx.x >= wblocks;
-    const int i = (bias ? (int)blockIdx.x - wblocks : (int)blockIdx.x) * 32 + e;
-    const int n = bias ? Cout : Cout * K;
-    const size_t stride = bias ? (size_t)Cout : (size_t)Cout * Kp;
-    const size_t at = bias ? (size_t)i : (size_t)(i / K) * Kp + i % K;
-    float v = 0.f;
-    if (i < n) {
-        const float *p = (bias ? bpart : part) + at;
-#pragma unroll 16
-        for (int c = q; c < nparts; c += kSumWays) v += p[(size_t)c * stride];
-    }
-    s[q][e] = v;
-    __syncthreads();
-    if (q == 0 && i < n) {
-        float r = s[0][e];
-        for (int k = 1; k < kSumWays; ++k) r += s[k][e];
-        float *o = bias ? gb : gw;
-        o[at] += r;
+    const int e = threadIdx.x & 31;
+    if ((int)blockIdx.x < wblocks) {
+        const int i = (int)blockIdx.x * 32 + e;
+        const size_t at = (size_t)(i / K) * Kp + i % K;
+        sum_parts<Plain>(part + at, gw + at, s, nparts, (size_t)Cout * Kp, i < Cout * K);
+    } else {
+        const int i = ((int)blockIdx.x - wblocks) * 32 + e;
+        sum_parts<Pair>(bpart + i, gb + i, s, nparts, (size_t)Cout, i < Cout);
     }
 }
 
