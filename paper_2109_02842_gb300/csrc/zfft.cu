@@ -156,8 +156,66 @@ k_fft_strided(const float2 *__restrict__ in, const float2 *__restrict__ in2, flo
 
 // Direct DFT along the middle axis with an explicit phase matrix:
 //   out[b][r][i] = scale * sum_{n < n_in} in[b][n][i] * T[r][n]
-// 32 rows x 64 columns per block of 128 threads, 4 x 4 outputs each: four
-// 16-byte shared loads feed 64 FMA (one output column a thread took five
+// in two kernels. A 32 x 32 output tile per block of 256 threads, 4 rows of one
+// column each, for few columns and few blocks (the rule is at the launch):
+__global__ void __launch_bounds__(256)
+k_dft_narrow(const float2 *__restrict__ in, const float2 *__restrict__ in2, float2 *__restrict__ out,
+              int n_in, int I, int out_rows, const float2 *__restrict__ T, float scale,
+              int out_bf16) {
+    __shared__ float2 xs[32][33];
+    __shared__ float2 ts[32][33];
+    const int tx = threadIdx.x & 31;
+    const int ty = threadIdx.x >> 5;   // 0..7
+    const int i = blockIdx.x * 32 + tx;
+    const int r0 = blockIdx.y * 32;
+    const size_t b = blockIdx.z;
+    float2 acc[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[q] = make_float2(0.f, 0.f);
+    for (int n0 = 0; n0 < n_in; n0 += 32) {
+        for (int q = 0; q < 4; ++q) {
+            const int nn = ty * 4 + q;
+            const int n = n0 + nn;
+            float2 x = make_float2(0.f, 0.f);
+            if (n < n_in && i < I) {
+                const size_t o = (b * n_in + n) * (size_t)I + i;
+                x = in[o];
+                if (in2) x = cadd(x, in2[o]);
+            }
+            xs[nn][tx] = x;
+            const int rr = r0 + ty * 4 + q;
+            ts[ty * 4 + q][tx] = (rr < out_rows && n0 + tx < n_in)
+                                     ? T[(size_t)rr * n_in + n0 + tx] : make_float2(0.f, 0.f);
+        }
+        __syncthreads();
+#pragma unroll 8
+        for (int nn = 0; nn < 32; ++nn) {
+            const float2 x = xs[nn][tx];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float2 t = ts[ty * 4 + q][nn];
+                acc[q].x += x.x * t.x - x.y * t.y;
+                acc[q].y += x.x * t.y + x.y * t.x;
+            }
+        }
+        __syncthreads();
+    }
+    if (i < I) {
+        for (int q = 0; q < 4; ++q) {
+            const int r = r0 + ty * 4 + q;
+            if (r >= out_rows) continue;
+            const float2 v = cscale(acc[q], scale);
+            const size_t o = (b * out_rows + r) * (size_t)I + i;
+            if (out_bf16)
+                reinterpret_cast<__nv_bfloat162 *>(out)[o] = __floats2bfloat162_rn(v.x, v.y);
+            else
+                out[o] = v;
+        }
+    }
+}
+
+// ... and 32 rows x 64 columns per block of 128 threads, 4 x 4 outputs each: four
+// 16-byte shared loads feed 64 FMA (one output column a thread takes five
 // 8-byte loads for 16). FP32 scan of 225 bins, 96 heights, 120 x 101 pixels:
 // 1041 -> 1027 us.
 constexpr int kDftK = 32, kDftRows = 32, kDftCols = 64;
@@ -260,8 +318,22 @@ cudaError_t launch_fft_strided(const float2 *in, float2 *out, int batch, int n_i
 cudaError_t launch_dft_strided(const float2 *in, float2 *out, int batch, int n_in, int I,
                                int out_rows, const float2 *T, float scale, cudaStream_t st,
                                const float2 *in2, int bf16_out) {
-    dim3 grid((I + kDftCols - 1) / kDftCols, (out_rows + kDftRows - 1) / kDftRows, batch);
-    k_dft_strided<<<grid, 128, 0, st>>>(in, in2, out, n_in, I, out_rows, T, scale, bf16_out);
+    // The wide tile costs 1.7 narrow ones, so it wins where it takes fewer than
+    // 1 / 1.7 of the narrow tile's blocks, and once its blocks (four warps of long
+    // chains) fill the device about three times. Narrow and wide, us: 127 points,
+    // 256 transforms of 32 columns 39.6 and 57.6, of 64 73.5 and 65.7, of 80 106
+    // and 109, of 128 136 and 114; 64 transforms of 64 24.9 and 24.7; 251 points
+    // onto 128 rows, 2304 columns 26.7 and 34.9, 4096 45.6 and 45.4, 9216 83.6 and
+    // 67.9.
+    const long long rows = (long long)((out_rows + kDftRows - 1) / kDftRows) * batch;
+    const int wide = (I + kDftCols - 1) / kDftCols, narrow = (I + 31) / 32;
+    if (17LL * wide < 10LL * narrow && rows * wide >= 400) {
+        dim3 grid(wide, (out_rows + kDftRows - 1) / kDftRows, batch);
+        k_dft_strided<<<grid, 128, 0, st>>>(in, in2, out, n_in, I, out_rows, T, scale, bf16_out);
+    } else {
+        dim3 grid(narrow, (out_rows + 31) / 32, batch);
+        k_dft_narrow<<<grid, 256, 0, st>>>(in, in2, out, n_in, I, out_rows, T, scale, bf16_out);
+    }
     return cudaGetLastError();
 }
 
