@@ -173,6 +173,10 @@ k_exact_sum(ExactDesc e, const float2 *__restrict__ S, const float2 *__restrict_
 // grows no further. 120 channels, 48 positions, 51 frequencies, 64^3 voxels:
 // 43.6 -> 14.3 ms (7.9 ms at the FP32 peak; the rest is the two phases of each
 // (voxel, channel, position), 16.2 ms with unpacked FMA).
+//
+// LINES: the 128 voxels of a warp are consecutive over the whole volume, each
+// with its own height, for planes of so few pixels that most lanes of a plane's
+// block would repeat the last one (the rule is at the launch).
 constexpr int kDirWarps = 8, kDirPx = 128, kDirTerms = 256, kDirPoly = 128;
 
 using bp::f2;
@@ -189,20 +193,36 @@ __device__ __forceinline__ ff ff_sqrt_sum(ff x, ff y) {
     return {r, (fmaf(-r, r, s.hi) + lo) * (0.5f * q)};
 }
 
-template <int MODE>
+template <int MODE, bool LINES>
 __global__ void __launch_bounds__(32 * kDirWarps, 3)
 k_bp_direct_uniform(DirectDesc e, const float2 *__restrict__ s, const float4 *__restrict__ chff,
                     const float2 *__restrict__ zs, const float2 *__restrict__ kff,
                     float2 *__restrict__ img) {
     __shared__ float4 sm_coef[kDirWarps * kDirTerms];   // [warp][term] {re, re, im, im}
-    __shared__ float2 sm_dz2[kDirWarps][32];            // (z - z'_n)^2 of the staged positions
+    // (z - z'_n)^2 of the staged positions; LINES: z'_n
+    __shared__ float2 sm_dz2[kDirWarps][32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float4 *coef = sm_coef + warp * kDirTerms;
-    const int np = e.nx * e.ny, px_blocks = (np + kDirPx - 1) / kDirPx;
-    const int iz = (int)(blockIdx.x / px_blocks);
-    const int pb = (int)(blockIdx.x - (unsigned)iz * px_blocks) * kDirPx;
-    const ff pz = ff_of(e.z0 + iz * e.dz);
+    const int np = e.nx * e.ny, px_blocks = LINES ? 1 : (np + kDirPx - 1) / kDirPx;
+    const int iz = LINES ? 0 : (int)(blockIdx.x / px_blocks);
+    // this block's first pixel of plane iz (LINES: 0, of the voxels from v0 on)
+    // and where they end
+    const long long v0 = LINES ? (long long)blockIdx.x * kDirPx : (long long)iz * np;
+    const int pb = LINES ? 0 : (int)(blockIdx.x - (unsigned)iz * px_blocks) * kDirPx;
+    const int pe = LINES ? (int)min((long long)kDirPx, (long long)np * e.nz - v0) : np;
     const int p0 = pb + lane;
+    ff pz[LINES ? 4 : 1];
+    int pixel[LINES ? 4 : 1];
+    if (LINES) {
+#pragma unroll
+        for (int k = 0; k < (LINES ? 4 : 1); ++k) {
+            const long long v = v0 + min(p0 + 32 * k, pe - 1);
+            pixel[k] = (int)(v % np);
+            pz[k] = ff_of(e.z0 + (double)(v / np) * e.dz);
+        }
+    } else {
+        pz[0] = ff_of(e.z0 + iz * e.dz);
+    }
     const int rows = e.n_f > kDirPoly ? 1 : min(32, kDirTerms / e.n_f);  // positions staged at a time
     // frequency of staged term `lane`, and its step over 32 terms (modulo n_f)
     const int lane_m = lane % e.n_f, step_m = 32 % e.n_f;
@@ -212,7 +232,8 @@ k_bp_direct_uniform(DirectDesc e, const float2 *__restrict__ s, const float4 *__
         ff rho_t[4], rho_r[MODE == 1 ? 4 : 1];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const int p = min(p0 + 32 * k, np - 1);          // past the image: the last pixel
+            // (past the image: the last pixel)
+            const int p = LINES ? pixel[LINES ? k : 0] : min(p0 + 32 * k, np - 1);
             const ff px = ff_of(e.x0 + (p % e.nx) * e.dx), py = ff_of(e.y0 + (p / e.nx) * e.dy);
             const ff dxt = ff_add(px, ff_neg({t.x, t.y})), dyt = ff_add(py, ff_neg({t.z, t.w}));
             rho_t[k] = ff_add(ff_sqr(dxt), ff_sqr(dyt));
@@ -239,15 +260,17 @@ k_bp_direct_uniform(DirectDesc e, const float2 *__restrict__ s, const float4 *__
                 }
                 if (lane < nr) {
                     const float2 zn = zs[n0 + lane];
-                    const ff d = ff_sqr(ff_add(pz, ff_neg({zn.x, zn.y})));
-                    sm_dz2[warp][lane] = make_float2(d.hi, d.lo);
+                    const ff d = ff_sqr(ff_add(pz[0], ff_neg({zn.x, zn.y})));
+                    sm_dz2[warp][lane] = LINES ? zn : make_float2(d.hi, d.lo);
                 }
                 __syncwarp();
                 for (int n = 0; n < nr; ++n) {
-                    const ff dz2 = {sm_dz2[warp][n].x, sm_dz2[warp][n].y};
+                    ff dz2 = {sm_dz2[warp][n].x, sm_dz2[warp][n].y};
+                    const ff zn = ff_neg(dz2);
                     float cs[4], sn[4], c0[4], s0[4];
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
+                        if (LINES) dz2 = ff_sqr(ff_add(pz[LINES ? k : 0], zn));
                         ff a = ff_sqrt_sum(rho_t[k], dz2);
                         a = MODE == 0 ? ff{a.hi + a.hi, a.lo + a.lo}
                                       : ff_add(a, ff_sqrt_sum(rho_r[MODE == 1 ? k : 0], dz2));
@@ -290,14 +313,13 @@ k_bp_direct_uniform(DirectDesc e, const float2 *__restrict__ s, const float4 *__
     }
     __syncthreads();
     for (int i = threadIdx.x; i < kDirPx; i += 32 * kDirWarps) {
-        const int p = pb + i;
-        if (p >= np) break;
+        if (pb + i >= pe) break;
         float2 g = part[i];
         for (int w = 1; w < kDirWarps; ++w) {
             g.x += part[w * kDirPx + i].x;
             g.y += part[w * kDirPx + i].y;
         }
-        img[(size_t)iz * np + p] = g;
+        img[v0 + pb + i] = g;
     }
 }
 
@@ -361,8 +383,19 @@ cudaError_t launch_exact_sum(const ExactDesc &e, const float2 *S, const float2 *
 cudaError_t launch_bp_direct(const DirectDesc &e, const float2 *s, const float4 *chff,
                              const float2 *zs, const float2 *kff, float2 *img, cudaStream_t st) {
     if (e.uniform) {
-        auto kern = e.mode == 1 ? k_bp_direct_uniform<1> : k_bp_direct_uniform<0>;
-        const unsigned blocks = (unsigned)((e.nx * e.ny + kDirPx - 1) / kDirPx) * (unsigned)e.nz;
+        // planes of up to 64 pixels, half a block, as lines, once there are more
+        // planes than SMs. Planes and lines, ms (120 channels, 48 positions, 51
+        // frequencies): 1 x 1 x 16384 voxels 109 and 1.39, 5 x 5 x 8192 54.8 and
+        // 11.9, 6 x 7 x 8192 54.8 and 19.3, 2 x 2 x 256 2.22 and 1.39, 5 x 5 x 128
+        // 1.35 and 1.40.
+        const int np = e.nx * e.ny;
+        const bool lines = np <= kDirPx / 2 && e.nz > 152;
+        auto kern = lines ? (e.mode == 1 ? k_bp_direct_uniform<1, true> : k_bp_direct_uniform<0, true>)
+                          : (e.mode == 1 ? k_bp_direct_uniform<1, false> : k_bp_direct_uniform<0, false>);
+        const long long blocks_ll = lines ? ((long long)np * e.nz + kDirPx - 1) / kDirPx
+                                          : (long long)((np + kDirPx - 1) / kDirPx) * e.nz;
+        if (blocks_ll > 0x7fffffffLL) return cudaErrorInvalidValue;
+        const unsigned blocks = (unsigned)blocks_ll;
         kern<<<blocks, 32 * kDirWarps, 0, st>>>(e, s, chff, zs, kff, img);
         return cudaGetLastError();
     }
