@@ -479,7 +479,9 @@ pl_status pl_batch_destroy(pl_batch *batch);
  *   (dz-1, dy-1, dx-1), zero padding; x BF16 [V][Cin]; w BF16
  *   [Cout][pl_nn_padded_k(Cin)] (row tail zero); bias FP32 [Cout] or NULL;
  *   relu != 0 applies max(., 0); out BF16 (out_bf16 != 0) or FP32 [V][Cout].
- *   BF16 tensor-core MMA with FP32 accumulation.
+ *   BF16 tensor-core MMA with FP32 accumulation. Any address that suits the
+ *   element type will do for x, w and out; the fast kernels take 16-byte
+ *   aligned ones (any x, and w 4-byte aligned, for Cin of 1 to 4).
  * pl_nn_conv3d_wgrad: gw[co][tap Cin + ci] += sum_v gy[v][co] x[v+off][ci] and
  *   gb[co] += sum_v gy[v][co] (gb may be NULL); x, gy BF16; gw, gb FP32;
  *   Cout <= 32, 49-64 or 113-128. `work` is caller-owned device scratch of at

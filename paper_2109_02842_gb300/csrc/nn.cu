@@ -16,8 +16,8 @@
 // below, BF16 mma.sync m16n8k16 with FP32 accumulation. All sum in the same
 // order, K in steps of 16, with equal results bit for bit. A block of 4
 // warps owns 64 voxels x (8 NT) output channels; per 16-wide K chunk it
-// stages the A tile (one 32-byte row per voxel when Cin is a multiple of 16,
-// an element gather otherwise) and the B tile in shared memory.
+// stages the A tile (one 32-byte row per voxel when Cin is a multiple of 16 and x
+// 16-byte aligned, an element gather otherwise) and the B tile in shared memory.
 // The backward pass reuses the forward kernel for the input gradient (the
 // transposed convolution is a convolution with flipped taps and swapped
 // channel roles); the weight gradient is in nn_wgrad.cu.
@@ -62,7 +62,7 @@ template <int NT, bool OUT_BF16>
 __global__ void __launch_bounds__(128)
 k_conv3d(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__restrict__ w,
          const float *__restrict__ bias, void *__restrict__ out, Vol vol, int Cin, int Cout,
-         int Kp, int relu) {
+         int Kp, int relu, bool xvec, bool wvec) {
     constexpr int NTILE = 8 * NT;
     __shared__ __align__(16) __nv_bfloat16 As[64][kRowPad];
     __shared__ __align__(16) __nv_bfloat16 Bs[NTILE][kRowPad];
@@ -72,14 +72,13 @@ k_conv3d(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__restrict__ 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, t = lane & 3;
     const int K = 27 * Cin;
-    const bool vec = (Cin % 16) == 0;
     float acc[NT][4];
 #pragma unroll
     for (int j = 0; j < NT; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
 
     for (int k0 = 0; k0 < Kp; k0 += 16) {
         // A tile: 64 voxels x 16 k
-        if (vec) {
+        if (xvec) {
             const int row = threadIdx.x >> 1, half = threadIdx.x & 1;
             const int tap = k0 / Cin, ci0 = k0 - tap * Cin;
             uint4 val = make_uint4(0u, 0u, 0u, 0u);
@@ -101,12 +100,19 @@ k_conv3d(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__restrict__ 
             }
         }
         // B tile: NTILE output channels x 16 k (k contiguous per channel)
-        for (int e = threadIdx.x; e < NTILE * 2; e += 128) {
-            const int n = e >> 1, half = e & 1;
-            uint4 val = make_uint4(0u, 0u, 0u, 0u);
-            if (n0 + n < Cout)
-                val = *reinterpret_cast<const uint4 *>(w + (size_t)(n0 + n) * Kp + k0 + 8 * half);
-            *reinterpret_cast<uint4 *>(&Bs[n][8 * half]) = val;
+        if (wvec) {
+            for (int e = threadIdx.x; e < NTILE * 2; e += 128) {
+                const int n = e >> 1, half = e & 1;
+                uint4 val = make_uint4(0u, 0u, 0u, 0u);
+                if (n0 + n < Cout)
+                    val = *reinterpret_cast<const uint4 *>(w + (size_t)(n0 + n) * Kp + k0 + 8 * half);
+                *reinterpret_cast<uint4 *>(&Bs[n][8 * half]) = val;
+            }
+        } else {
+            for (int e = threadIdx.x; e < NTILE * 16; e += 128) {
+                const int n = e >> 4, k = e & 15;
+                Bs[n][k] = n0 + n < Cout ? w[(size_t)(n0 + n) * Kp + k0 + k] : __float2bfloat16(0.f);
+            }
         }
         __syncthreads();
         unsigned a[4];
@@ -506,18 +512,20 @@ cudaError_t nn_conv3d(const void *x, const void *w, const float *bias, void *out
     Vol vol{D, H, W};
     const auto *xb = (const __nv_bfloat16 *)x;
     const auto *wb = (const __nv_bfloat16 *)w;
+    // 16-byte loads where they are aligned, else single elements
+    const bool xv = Cin % 16 == 0 && (uintptr_t)x % 16 == 0, wv = (uintptr_t)w % 16 == 0;
     if (Cout <= 8) {
         dim3 grid((V + 63) / 64, (Cout + 7) / 8);
-        if (out_bf16) k_conv3d<1, true><<<grid, 128, 0, st>>>(xb, wb, bias, out, vol, Cin, Cout, Kp, relu);
-        else k_conv3d<1, false><<<grid, 128, 0, st>>>(xb, wb, bias, out, vol, Cin, Cout, Kp, relu);
+        if (out_bf16) k_conv3d<1, true><<<grid, 128, 0, st>>>(xb, wb, bias, out, vol, Cin, Cout, Kp, relu, xv, wv);
+        else k_conv3d<1, false><<<grid, 128, 0, st>>>(xb, wb, bias, out, vol, Cin, Cout, Kp, relu, xv, wv);
     } else if (Cout <= 16) {
         dim3 grid((V + 63) / 64, (Cout + 15) / 16);
-        if (out_bf16) k_conv3d<2, true><<<grid, 128, 0, st>>>(xb, wb, bias, out, vol, Cin, Cout, Kp, relu);
-        else k_conv3d<2, false><<<grid, 128, 0, st>>>(xb, wb, bias, out, vol, Cin, Cout, Kp, relu);
+        if (out_bf16) k_conv3d<2, true><<<grid, 128, 0, st>>>(xb, wb, bias, out, vol, Cin, Cout, Kp, relu, xv, wv);
+        else k_conv3d<2, false><<<grid, 128, 0, st>>>(xb, wb, bias, out, vol, Cin, Cout, Kp, relu, xv, wv);
     } else {
         dim3 grid((V + 63) / 64, (Cout + 31) / 32);
-        if (out_bf16) k_conv3d<4, true><<<grid, 128, 0, st>>>(xb, wb, bias, out, vol, Cin, Cout, Kp, relu);
-        else k_conv3d<4, false><<<grid, 128, 0, st>>>(xb, wb, bias, out, vol, Cin, Cout, Kp, relu);
+        if (out_bf16) k_conv3d<4, true><<<grid, 128, 0, st>>>(xb, wb, bias, out, vol, Cin, Cout, Kp, relu, xv, wv);
+        else k_conv3d<4, false><<<grid, 128, 0, st>>>(xb, wb, bias, out, vol, Cin, Cout, Kp, relu, xv, wv);
     }
     return cudaGetLastError();
 }
