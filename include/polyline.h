@@ -253,7 +253,9 @@ enum {
  *                        lo = BF16(S - hi) (lo planes unused with precision 2)
  *  PL_WS_RT_OPERAND_E -> the plan-time factor [n_pad][re hi, re lo, im hi,
  *                        im lo][Lp][Kp], E[u][i][m] = alpha_um
- *                        e^{j theta_um (i - L/2)}, b[c][i][u] = sum_m S E */
+ *                        e^{j theta_um (i - L/2)}, b[c][i][u] = sum_m S E
+ * With more than 128 frequencies each real number has three such parts instead
+ * of two: [n_pad][re 0, re 1, re 2, im 0, im 1, im 2][...], whose sum it is. */
 enum { PL_WS_RT_OPERAND_A = 16, PL_WS_RT_OPERAND_E = 17 };
 
 /* Create a plan: validates the inputs, allocates device workspace on the

@@ -14,7 +14,8 @@ cudaError_t launch_fft_strided(const float2 *in, float2 *out, int batch, int n_i
                                const FftPlan &plan, const float2 *tw, int sgn, float scale,
                                int out_rows, int out_off, cudaStream_t st,
                                void *split_A = nullptr, int split_Kp = 0,
-                               const float2 *in2 = nullptr, int ld = 0, int bf16_out = 0);
+                               const float2 *in2 = nullptr, int ld = 0, int bf16_out = 0,
+                               int split_limbs = 2);
 // (ld: row stride in elements, 0 = I; a launch may cover columns [0, I) of
 // wider rows, the pointers offset by the first column)
 // in2 (optional): a second input of the same shape, added to `in` on load
@@ -212,6 +213,7 @@ struct RtTcArgs {
     int C, Np, M;
     int Kp;              // frequencies rounded up to 64 (the K of the products)
     int natoms;          // Kp / 64
+    int limbs;           // BF16 parts of each real operand: 2 (hi, lo), or 3 with 3 or 4 atoms
     int L, Lp;           // table rows; rounded up to 16
     int nh, Lh;          // row parts per bin (blocks along the rows) and rows per part,
                          // a multiple of 16 (the N of the products)
@@ -224,10 +226,12 @@ struct RtTcArgs {
                          // wait on a barrier nothing completes
 };
 size_t range_table_tc_smem_bytes(const RtTcArgs &ra);
-// E [N_p][re hi, re lo, im hi, im lo][Lp][Kp] BF16: alpha_um e^{+j theta_um (i - L/2)}
+int range_table_tc_max_rows(int limbs);
+// E [N_p][re parts, im parts][Lp][Kp] BF16: alpha_um e^{+j theta_um (i - L/2)}
 cudaError_t launch_setup_rt_E(const NufftDesc &d, double dz, const double *k, const double *kc,
-                              const float2 *alpha, int Lp, int Kp, void *E, cudaStream_t st);
-// S -> A (scratch [N_p][4][C][Kp] BF16; skipped when `prepared`: the
+                              const float2 *alpha, int Lp, int Kp, int limbs, void *E,
+                              cudaStream_t st);
+// S -> A (scratch [N_p][2 limbs][C][Kp] BF16; skipped when `prepared`: the
 // z-FFT wrote A) -> prod (scratch [N_p][2][nh * Lh][C rounded up to 128] uint32) -> table
 // [C][2][L][row_words uint32]
 cudaError_t launch_range_table_tc(const RtTcArgs &ra, const CUtensorMap &tmA,

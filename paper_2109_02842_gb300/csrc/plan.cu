@@ -822,6 +822,7 @@ pl_status build_plan(pl_plan *P, const pl_geometry *g, const pl_scan *s, const p
         ra.M = P->M;
         ra.Kp = (P->M + 63) / 64 * 64;
         ra.natoms = ra.Kp / 64;
+        ra.limbs = ra.natoms > 2 ? 3 : 2;
         ra.L = L;
         ra.Lp = (L + 15) / 16 * 16;
         // the fewest row parts whose two operand buffers (the persistent
@@ -829,7 +830,8 @@ pl_status build_plan(pl_plan *P, const pl_geometry *g, const pl_scan *s, const p
         // accumulator pairs fit in TMEM
         for (ra.nh = 1;; ++ra.nh) {
             ra.Lh = ((ra.Lp + ra.nh - 1) / ra.nh + 15) / 16 * 16;
-            if ((range_table_tc_smem_bytes(ra) <= 227 * 1024 && 4 * ra.Lh <= 512) || ra.Lh <= 16)
+            if ((range_table_tc_smem_bytes(ra) <= 227 * 1024 &&
+                 ra.Lh <= range_table_tc_max_rows(ra.limbs)) || ra.Lh <= 16)
                 break;
         }
         ra.idesc = tc05::idesc_bf16(128, ra.Lh, 0);
@@ -844,20 +846,20 @@ pl_status build_plan(pl_plan *P, const pl_geometry *g, const pl_scan *s, const p
             ra.grid = sms;
         }
         // three and four atoms (129 to 256 frequencies) only with the FP32
-        // spectrum and the hi/lo split, where sums and NUFFT agree to FP32
-        // rounding (through a table rounded to BF16 the two differ by more),
-        // and from 16384 (channel, bin) pairs on. Table stage, NUFFT and sums,
-        // ms: 201 frequencies, 115 channels, 216 bins 0.351 and 0.058; 256, 576,
-        // 512: 4.82 and 0.372; 160, 128, 128: 0.125 and 0.031. (160, 64, 64:
-        // 0.033 and 0.020; the parity tests hold plans of that size to the
-        // NUFFT-built table.)
+        // spectrum and the hi/lo split, where the sums (their operands in three
+        // BF16 parts) are as close to 64 bits as the NUFFT (through a table
+        // rounded to BF16 the two differ by more), and from 16384 (channel, bin)
+        // pairs on. Table stage, NUFFT and sums, us: 201 frequencies, 115 channels,
+        // 216 bins 131 and 50; 384 x 200 389 and 88; 160 frequencies, 128 x 128 66
+        // and 28. (160 frequencies, 64 x 64: 33 and 20 with two parts; the parity
+        // tests hold plans of that size to the NUFFT-built table.)
         const bool natoms_ok = ra.natoms <= 2 || (ra.natoms <= 4 && P->precision == 0 &&
                                                   (long long)P->C * P->Np >= 16384);
-        P->rt_tc = natoms_ok && ra.Lp <= 256 && 4 * ra.Lh <= 512 &&
+        P->rt_tc = natoms_ok && ra.Lp <= 256 && ra.Lh <= range_table_tc_max_rows(ra.limbs) &&
                    range_table_tc_smem_bytes(ra) <= 227 * 1024;
         if (P->rt_tc) {
-            const size_t nE = (size_t)P->Np * 4 * ra.Lp * ra.Kp;
-            const size_t nA = (size_t)P->Np * 4 * P->C * ra.Kp;
+            const size_t nE = (size_t)P->Np * 2 * ra.limbs * ra.Lp * ra.Kp;
+            const size_t nA = (size_t)P->Np * 2 * ra.limbs * P->C * ra.Kp;
             const size_t nprod = (size_t)P->Np * 2 * ra.nh * ra.Lh * ((P->C + 127) / 128 * 128);
             PL_CUDA(plan_malloc(&P->d_rtE, nE * 2), "cudaMalloc");
             PL_CUDA(plan_malloc(&P->d_rtA, nA * 2), "cudaMalloc");
@@ -865,12 +867,14 @@ pl_status build_plan(pl_plan *P, const pl_geometry *g, const pl_scan *s, const p
             PL_CUDA(plan_malloc(&P->d_rtprod, nprod * 4), "cudaMalloc");
             ws += nE * 2 + nA * 2 + nprod * 4;
             PL_CUDA(launch_setup_rt_E(d, P->dzs, P->d_k, P->d_kc, P->d_alpha, ra.Lp, ra.Kp,
-                                      P->d_rtE, st),
+                                      ra.limbs, P->d_rtE, st),
                     "setup_rt_E");
-            const cuuint64_t da[3] = {(cuuint64_t)ra.Kp, (cuuint64_t)P->C, 4 * (cuuint64_t)P->Np};
+            const cuuint64_t da[3] = {(cuuint64_t)ra.Kp, (cuuint64_t)P->C,
+                                      2 * ra.limbs * (cuuint64_t)P->Np};
             const cuuint64_t sa[2] = {(cuuint64_t)ra.Kp * 2, (cuuint64_t)P->C * ra.Kp * 2};
             const cuuint32_t ba[3] = {64, 128, 1};
-            const cuuint64_t db[3] = {(cuuint64_t)ra.Kp, (cuuint64_t)ra.Lp, 4 * (cuuint64_t)P->Np};
+            const cuuint64_t db[3] = {(cuuint64_t)ra.Kp, (cuuint64_t)ra.Lp,
+                                      2 * ra.limbs * (cuuint64_t)P->Np};
             const cuuint64_t sb[2] = {(cuuint64_t)ra.Kp * 2, (cuuint64_t)ra.Lp * ra.Kp * 2};
             const cuuint32_t bb[3] = {64, (cuuint32_t)ra.Lh, 1};
             const cuuint32_t e3[3] = {1, 1, 1};
@@ -932,7 +936,8 @@ static pl_status stage_zfft(pl_plan *P, const float2 *echo, cudaStream_t st, boo
     const int bf16 = P->precision == 2 ? 1 : 0;
     if (P->fwd_fft && split)      // straight into the tensor-core range table's operand
         PL_CUDA(launch_fft_strided(echo, P->d_S, P->C, P->N, P->M, P->zplan, P->d_twz, -1, 1.0f,
-                                   P->Np, 0, st, P->d_rtA, P->rt.Kp, nullptr, 0, bf16), "zfft");
+                                   P->Np, 0, st, P->d_rtA, P->rt.Kp, nullptr, 0, bf16,
+                                   P->rt.limbs), "zfft");
     else if (P->fwd_fft)
         PL_CUDA(launch_fft_strided(echo, P->d_S, P->C, P->N, P->M, P->zplan, P->d_twz, -1, 1.0f,
                                    P->Np, 0, st, nullptr, 0, nullptr, 0, s_bf16), "zfft");
@@ -1508,10 +1513,10 @@ pl_status pl_plan_workspace(pl_plan *P, int stage, void **dev_ptr, size_t *bytes
             if (!(P->block_config == 4 && P->rt_tc)) break;
             if (stage == PL_WS_RT_OPERAND_A) {
                 *dev_ptr = P->d_rtA;
-                *bytes = (size_t)P->Np * 4 * P->C * P->rt.Kp * 2;
+                *bytes = (size_t)P->Np * 2 * P->rt.limbs * P->C * P->rt.Kp * 2;
             } else {
                 *dev_ptr = P->d_rtE;
-                *bytes = (size_t)P->Np * 4 * P->rt.Lp * P->rt.Kp * 2;
+                *bytes = (size_t)P->Np * 2 * P->rt.limbs * P->rt.Lp * P->rt.Kp * 2;
             }
             return PL_OK;
         case PL_STAGE_BACKPROJECT:

@@ -37,6 +37,7 @@ struct SplitOut {
     __nv_bfloat16 *A;        // nullptr: plain output
     int batch, Kp;
     int hi_only;             // split output: hi planes only (BF16 spectrum)
+    int limbs;               // split output: BF16 parts of a real number (2 or 3)
     int bf16_rows;           // plain output as bfloat16 (re, im) pairs
 };
 // The FFT stages run on column pairs (float4 shared-memory accesses, a zero
@@ -108,6 +109,22 @@ k_fft_strided(const float2 *__restrict__ in, const float2 *__restrict__ in2, flo
             if (r < 0) r += N;
             if (r >= out_rows || i0 + 2 * cp >= I) return;
             const float2 v0 = cscale(x0, scale), v1 = cscale(x1, scale);
+            if (sp.limbs == 3) {
+                __nv_bfloat16 *o = A + (size_t)r * 6 * plane + 2 * cp;
+                float re0 = v0.x, re1 = v1.x, im0 = v0.y, im1 = v1.y;
+#pragma unroll
+                for (int l = 0; l < 3; ++l, o += plane) {
+                    const __nv_bfloat162 re = __floats2bfloat162_rn(re0, re1);
+                    const __nv_bfloat162 im = __floats2bfloat162_rn(im0, im1);
+                    *reinterpret_cast<__nv_bfloat162 *>(o) = re;
+                    *reinterpret_cast<__nv_bfloat162 *>(o + 3 * plane) = im;
+                    re0 -= __low2float(re);
+                    re1 -= __high2float(re);
+                    im0 -= __low2float(im);
+                    im1 -= __high2float(im);
+                }
+                return;
+            }
             const __nv_bfloat16 h0 = __float2bfloat16(v0.x), h1 = __float2bfloat16(v1.x);
             const __nv_bfloat16 g0 = __float2bfloat16(v0.y), g1 = __float2bfloat16(v1.y);
             __nv_bfloat16 *o = A + (size_t)r * 4 * plane + 2 * cp;
@@ -290,7 +307,7 @@ cudaError_t launch_fft_strided(const float2 *in, float2 *out, int batch, int n_i
                                const FftPlan &plan, const float2 *tw, int sgn, float scale,
                                int out_rows, int out_off, cudaStream_t st,
                                void *split_A, int split_Kp, const float2 *in2, int ld,
-                               int bf16_out) {
+                               int bf16_out, int split_limbs) {
     const size_t smem = fft_strided_smem_bytes(plan.n);
     // copies of column pairs need 16-byte aligned rows: I even, 16-byte aligned
     // buffers; the split output always takes pairs (operand rows of Kp, a
@@ -308,7 +325,7 @@ cudaError_t launch_fft_strided(const float2 *in, float2 *out, int batch, int n_i
     if (e != cudaSuccess) return e;
     dim3 grid((I + kFftIB - 1) / kFftIB, batch);
     // bf16_out: with split_A, the hi planes only; else bfloat16 (re, im) rows
-    const SplitOut sp{(__nv_bfloat16 *)split_A, batch, split_Kp, split_A ? bf16_out : 0,
+    const SplitOut sp{(__nv_bfloat16 *)split_A, batch, split_Kp, split_A ? bf16_out : 0, split_limbs,
                       split_A ? 0 : bf16_out};
     kern<<<grid, kFftThreads, smem, st>>>(in, in2, out, n_in, I, ld, plan, tw, sgn, scale, out_rows, out_off,
                                   sp);
