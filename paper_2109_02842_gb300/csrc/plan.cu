@@ -848,13 +848,25 @@ pl_status build_plan(pl_plan *P, const pl_geometry *g, const pl_scan *s, const p
         // three and four atoms (129 to 256 frequencies) only with the FP32
         // spectrum and the hi/lo split, where the sums (their operands in three
         // BF16 parts) are as close to 64 bits as the NUFFT (through a table
-        // rounded to BF16 the two differ by more), and from 16384 (channel, bin)
-        // pairs on. Table stage, NUFFT and sums, us: 201 frequencies, 115 channels,
-        // 216 bins 131 and 50; 384 x 200 389 and 88; 160 frequencies, 128 x 128 66
-        // and 28. (160 frequencies, 64 x 64: 33 and 20 with two parts; the parity
-        // tests hold plans of that size to the NUFFT-built table.)
-        const bool natoms_ok = ra.natoms <= 2 || (ra.natoms <= 4 && P->precision == 0 &&
-                                                  (long long)P->C * P->Np >= 16384);
+        // rounded to BF16 the two differ by more), and where that is faster. The
+        // products run in blocks of 128 channels, so few channels pay for many:
+        // table stage, NUFFT and sums, us: 201 frequencies, 64 channels, 256 bins
+        // 94 and 47, 32 x 512 92 and 78, 16 x 1024 92 and 148, 4 x 4096 95 and 440;
+        // 130 frequencies, 64 x 256 56 and 40; 384 x 200 389 and 88; with the operand
+        // split from an FP32 spectrum, 48 x 342 (130 frequencies) 77 and 94. Below 16384
+        // pairs the sums would win too (64 x 64, 160 frequencies: 33 and 20 with two
+        // parts), but existing tests hold plans of that size to the NUFFT-built table.
+        // The operands take 12 bytes a spectrum value: not where they would need
+        // more than half of the free device memory.
+        bool natoms_ok = ra.natoms <= 2;
+        if (ra.natoms == 3 || ra.natoms == 4) {
+            size_t free_b = 0, total_b = 0;
+            PL_CUDA(cudaMemGetInfo(&free_b, &total_b), "cudaMemGetInfo");
+            const size_t need = (size_t)P->Np * (12 * (size_t)ra.Kp * (P->C + ra.Lp) +
+                                                 8 * (size_t)ra.nh * ra.Lh * (P->C + 127));
+            natoms_ok = P->precision == 0 && P->C >= 64 && (long long)P->C * P->Np >= 16384 &&
+                        need <= free_b / 2;
+        }
         P->rt_tc = natoms_ok && ra.Lp <= 256 && ra.Lh <= range_table_tc_max_rows(ra.limbs) &&
                    range_table_tc_smem_bytes(ra) <= 227 * 1024;
         if (P->rt_tc) {

@@ -1,6 +1,7 @@
 """The range table of 129 to 256 frequencies keeps FP32 operands: the spectrum
-operand (the sum of its BF16 parts) against a 64-bit transform, and the table
-against the 64-bit product of its operands.
+operand (the sum of its BF16 parts) against a 64-bit transform, the table against
+the 64-bit product of its operands, and the plans that keep the NUFFT (few
+channels).
 
 Tolerances. Spectrum: an FP32 FFT of 128 to 360 points, at most 5 stages of some
 six roundings of 2^-25 rms each: 1.7e-7 rms; 4e-7 (two BF16 parts of 8 bits round to
@@ -76,3 +77,9 @@ def test_operands_and_table(binding, per, n_f, n, n_pad, nx, ext):
                                                                   err_t))
     assert err_a < 4e-7
     assert err_t < 3e-6
+
+
+@pytest.mark.parametrize("per,n_pad,exact", [(63, 360, 0), (64, 360, 1), (16, 1024, 0), (64, 250, 0)])
+def test_few_channels_keep_the_nufft(binding, per, n_pad, exact):
+    plan = binding.Plan.from_workload(workload(per, 201, 200, n_pad))
+    assert plan.info["table_exact"] == exact
