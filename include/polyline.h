@@ -357,7 +357,10 @@ pl_status pl_plan_get_info(const pl_plan *plan, pl_info *info);
  *  PL_STAGE_BACKPROJECT -> image spectrum G, complex64 [parts][n_pad][ny][nx]: the
  *                          spectrum is the sum over parts (the channel parts of the
  *                          planar block_config 4 layout where they are kept
- *                          apart, else 1) */
+ *                          apart, else 1). With more than two parts the first
+ *                          call synchronises the device and has later executions
+ *                          clear parts 1 and on once part 0 holds the sum; a graph
+ *                          captured before it does not clear them */
 pl_status pl_plan_workspace(pl_plan *plan, int stage, void **dev_ptr, size_t *bytes);
 
 /* Per-stage timing with CUDA events recorded on the execute stream.

@@ -59,8 +59,8 @@ bool zidft_tc_make_map(const ZidftTcArgs &a, const __nv_bfloat16 *tb, CUtensorMa
 size_t zidft_tc_smem_bytes(const ZidftTcArgs &a);
 cudaError_t launch_zidft_tc(const ZidftTcArgs &a, const CUtensorMap *map, const float2 *G,
                             const float2 *G2, float2 *out, int *err, cudaStream_t st);
-// G[0] += G[1] + ... + G[parts - 1], spectra of n values; the others are cleared
-cudaError_t launch_sum_spectra(float2 *G, int parts, size_t n, cudaStream_t st);
+// G[0] += G[1] + ... + G[parts - 1], spectra of n values; `clear`: the others are cleared
+cudaError_t launch_sum_spectra(float2 *G, int parts, size_t n, bool clear, cudaStream_t st);
 
 // ---- setup.cu --------------------------------------------------------------
 // Per k_z bin: kappa range over propagating frequencies; kc = centre (double

@@ -694,11 +694,18 @@ pl_status build_plan(pl_plan *P, const pl_geometry *g, const pl_scan *s, const p
         // added in order, so results stay bitwise reproducible. Whole scan: 64
         // channels, 32 x 32 pixels (16 -> 64 blocks) 59.4 -> 45.0 us (49.1 with
         // four parts), 120 channels, 64 x 64 (64 -> 128 blocks) 76 -> 67 us.
+        // Scenes of a batch share the SMs. Its persistent back-projection, whose
+        // layout one_block_per_sm is, fills them with two parts (twelve such scenes
+        // 366 and 390 us with more, twenty-four of 96 channels 467 and 513); scenes
+        // launched one by one give the bits of their plans alone, so they take the
+        // parts too: three and four small scenes gain (136 -> 130, 95 -> 94 us),
+        // twelve of 64 channels are even, twelve and twenty-four of 120 and 96
+        // channels lose 6 % (319 -> 337, 366 -> 389).
         // Up to 256 channels: the accumulation error of longer sums would
         // change with the split by more than 1e-5 of the image. Not with four
         // taps: such a plan makes the learned path's input, whose BF16
         // roundings carry a change of its last bits to 3e-4 of its image.
-        if (ta.nsplit == 2 && P->C <= 256 && W != 4) {
+        if (ta.nsplit == 2 && P->C <= 256 && W != 4 && !o.one_block_per_sm) {
             int dev = 0, sms = 0;
             PL_CUDA(cudaGetDevice(&dev), "cudaGetDevice");
             PL_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev),
@@ -1008,7 +1015,8 @@ pl_status pl_stage_backproject(pl_plan *P, cudaStream_t st) {
 static pl_status stage_zifft(pl_plan *P, float2 *image, cudaStream_t st, int parts) {
     const int P2 = P->grid.nx * P->grid.ny;
     if (parts > 2) {
-        PL_CUDA(launch_sum_spectra(P->d_G, parts, (size_t)P->Np * P2, st), "sum_spectra");
+        PL_CUDA(launch_sum_spectra(P->d_G, parts, (size_t)P->Np * P2, P->inspect_parts, st),
+                "sum_spectra");
         parts = 1;
     }
     const float2 *G2 = parts > 1 ? P->d_G + (size_t)P->Np * P2 : nullptr;
@@ -1532,6 +1540,14 @@ pl_status pl_plan_workspace(pl_plan *P, int stage, void **dev_ptr, size_t *bytes
             }
             return PL_OK;
         case PL_STAGE_BACKPROJECT:
+            if (g_parts(P) > 2 && !P->inspect_parts) {
+                // the first look: part 0 holds the sum of the executions so far
+                PL_CUDA(cudaDeviceSynchronize(), "workspace");
+                PL_CUDA(cudaMemset((char *)P->d_G + g_bytes(P), 0, (g_parts(P) - 1) * g_bytes(P)),
+                        "workspace");
+                PL_CUDA(cudaDeviceSynchronize(), "workspace");
+                P->inspect_parts = true;
+            }
             *dev_ptr = P->d_G;
             *bytes = (size_t)g_parts(P) * g_bytes(P);
             return PL_OK;

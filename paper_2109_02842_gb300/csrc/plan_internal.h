@@ -82,6 +82,9 @@ struct pl_plan {
     float2 *d_S = nullptr, *d_G = nullptr;
     void *d_table = nullptr;
     size_t table_bytes = 0;
+    // the spectra of more than two channel parts are looked at: parts 1 and on are
+    // cleared once they are in part 0 (see pl_plan_workspace)
+    bool inspect_parts = false;
     float2 *d_echo_in = nullptr, *d_img_out = nullptr;   // pl_execute_host staging
     // pl_execute_host_stream: a second staging pair, the copy streams and the
     // events that order them against the reconstruction
