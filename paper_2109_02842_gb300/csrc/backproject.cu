@@ -57,8 +57,7 @@ template <int UT, int W, int CC, int MINB, int PX>
 cudaError_t launch_t(const BpDesc &p, const CoefTable &ct, const void *table, const TileGeo *tgeo, const float2 *kc_hl,
                      float2 *G, cudaStream_t st) {
     const size_t smem = BpSmem<UT, W, CC>::bytes(p.R, p.n_chan, p.bf16);
-    cudaError_t e = cudaFuncSetAttribute(k_backproject<UT, W, CC, MINB, PX>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem(k_backproject<UT, W, CC, MINB, PX>, smem);
     if (e != cudaSuccess) return e;
     dim3 grid((p.nx + TX * PX - 1) / (TX * PX), (p.ny + TY - 1) / TY, (p.n_pad + UT - 1) / UT);
     k_backproject<UT, W, CC, MINB, PX><<<grid, TX * TY, smem, st>>>(p, ct, table, tgeo,

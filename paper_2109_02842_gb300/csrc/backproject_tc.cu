@@ -1239,8 +1239,7 @@ cudaError_t launch_t(const BpDesc &p, const CoefTable &ct, const TcArgs &ta, con
                      const TileGeo *tgeo, const float2 *kc_hl, float2 *G, int *err,
                      cudaStream_t st) {
     const size_t smem = backproject_tc_smem_bytes(ta);
-    cudaError_t e = cudaFuncSetAttribute(k_backproject_tc<W, KS, SPLIT, NPAR, PLANAR, CPR>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem(k_backproject_tc<W, KS, SPLIT, NPAR, PLANAR, CPR>, smem);
     if (e != cudaSuccess) return e;
     const int total = backproject_tc_blocks(p, ta);
     const int nblk = ta.nblk > 0 ? ta.nblk : total - ta.blk0;
@@ -1270,8 +1269,7 @@ cudaError_t launch_sp(const BpDesc &p, const CoefTable &ct, const TcArgs &ta, co
                       cudaStream_t st) {
     const size_t smem = backproject_tc_smem_bytes(ta);
     constexpr int NSET = 2;
-    cudaError_t e = cudaFuncSetAttribute(k_backproject_tc_sp<W, SPLIT, NPAR, NSET, RW, PLANAR>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem(k_backproject_tc_sp<W, SPLIT, NPAR, NSET, RW, PLANAR>, smem);
     if (e != cudaSuccess) return e;
     const int total = backproject_tc_blocks(p, ta);
     const int nblk = ta.nblk > 0 ? ta.nblk : total - ta.blk0;
@@ -1379,8 +1377,7 @@ cudaError_t launch_backproject_tc_batch(const TcBatchMaps &maps, const CoefTable
     if (n_scenes < 1 || n_scenes > kTcBatchMaxScenes || grid < 1 || smem > 227 * 1024)
         return cudaErrorInvalidValue;
     auto kern = split == 3 ? k_backproject_tc_batch<6, 3> : k_backproject_tc_batch<6, 1>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = allow_dynamic_smem(kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<grid, Warps<3>::threads, smem, st>>>(maps, ct, scenes, n_scenes, total, counters, err);
     return cudaGetLastError();

@@ -138,8 +138,7 @@ template <int UT, int CC, int MINB, int PX>
 cudaError_t launch_batch_t(const BatchConst &bc, const BatchScene *scenes, int *counters,
                            size_t smem, int *blocks_out, bool query, cudaStream_t st) {
     auto kern = k_batch<UT, CC, MINB, PX>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = allow_dynamic_smem(kern, smem);
     if (e != cudaSuccess) return e;
     if (query) {
         int per_sm = 0, dev = 0, sms = 0;

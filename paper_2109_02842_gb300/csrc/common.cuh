@@ -8,6 +8,19 @@
 #define PL_TWO_PI 6.283185307179586476925286766559
 
 // ---------------------------------------------------------------------------
+// Lets a kernel (of at most 1 KB static shared memory) take `bytes` of dynamic
+// shared memory. The limit set is the same whatever the size: with the size of
+// the call, a thread with a smaller plan could lower it between another thread's
+// call and its launch.
+// ---------------------------------------------------------------------------
+template <class Kernel>
+inline cudaError_t allow_dynamic_smem(Kernel kernel, size_t bytes) {
+    constexpr size_t most = 226 * 1024;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)(bytes > most ? bytes : most));
+}
+
+// ---------------------------------------------------------------------------
 // complex helpers (float2 = (re, im))
 // ---------------------------------------------------------------------------
 __host__ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {

@@ -349,9 +349,7 @@ cudaError_t launch_nt(const MmaShape &s, const __nv_bfloat16 *x, const __nv_bflo
                       const float *bias, void *out, int out_bf16, cudaStream_t st) {
     auto kern = out_bf16 ? k_conv3d_mma<NT, MT, true> : k_conv3d_mma<NT, MT, false>;
     const size_t smem = mma_smem(s);
-    // (the same limit whatever the shape: with this call's size, a thread with a
-    // smaller shape could lower it between another thread's call and launch)
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+    cudaError_t e = allow_dynamic_smem(kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<dim3(s.nx * s.ny * s.nz, s.n_co), kThreads, smem, st>>>(x, w, bias, out, s);
     return cudaGetLastError();

@@ -46,8 +46,7 @@ cudaError_t launch_ub(const NufftDesc &d, const FftPlan &fp, const float2 *S, co
                       const float *xg, const float *dec, const float2 *tw_fine, void *table,
                       int fmt, cudaStream_t st) {
     const size_t smem = range_table_smem_bytes(d);
-    cudaError_t e = cudaFuncSetAttribute(k_range_table<UB>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem(k_range_table<UB>, smem);
     if (e != cudaSuccess) return e;
     dim3 grid((d.n_pad + UB - 1) / UB, d.n_chan);
     k_range_table<UB><<<grid, 256, smem, st>>>(d, fp, S, alpha, xg, dec, tw_fine, table, fmt);

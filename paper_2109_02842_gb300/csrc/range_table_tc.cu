@@ -717,7 +717,7 @@ cudaError_t launch_range_table_tc(const RtTcArgs &ra, const CUtensorMap &tmA,
     }
     const size_t smem = range_table_tc_smem_bytes(ra);
     auto kern = ra.limbs == 3 ? k_range_table_tc3 : k_range_table_tc;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = allow_dynamic_smem(kern, smem);
     if (e != cudaSuccess) return e;
     // blocks take (channel block, bin) pairs with all their row parts; with
     // three parts, one row part of one

@@ -320,8 +320,7 @@ cudaError_t launch_fft_strided(const float2 *in, float2 *out, int batch, int n_i
                        ((uintptr_t)in2 % 16 == 0) && (split_A || (uintptr_t)out % 16 == 0);
     auto kern = split_A ? (pairs ? k_fft_strided<true, true> : k_fft_strided<false, true>)
                         : (pairs ? k_fft_strided<true, false> : k_fft_strided<false, false>);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = allow_dynamic_smem(kern, smem);
     if (e != cudaSuccess) return e;
     dim3 grid((I + kFftIB - 1) / kFftIB, batch);
     // bf16_out: with split_A, the hi planes only; else bfloat16 (re, im) rows

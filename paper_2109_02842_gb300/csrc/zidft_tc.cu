@@ -358,8 +358,7 @@ cudaError_t launch_zidft_tc(const ZidftTcArgs &a, const CUtensorMap *map, const 
     if (a.nzc < 16 || a.nzc > 96 || a.nzc % 16 || 2 * a.nzc + 64 > (int)kTmemCols)
         return cudaErrorInvalidValue;
     const size_t smem = zidft_tc_smem_bytes(a);
-    cudaError_t e = cudaFuncSetAttribute(k_zidft_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = allow_dynamic_smem(k_zidft_tc, smem);
     if (e != cudaSuccess) return e;
     const long long blocks = (long long)((a.n_cols + 127) / 128) * a.zchunks;
     k_zidft_tc<<<(unsigned)blocks, kThreads, smem, st>>>(*map, G, G2, out, a, err);
