@@ -37,16 +37,16 @@ struct SplitOut {
     __nv_bfloat16 *A;        // nullptr: plain output
     int batch, Kp;
     int hi_only;             // split output: hi planes only (BF16 spectrum)
-    int limbs;               // split output: BF16 parts of a real number (2 or 3)
     int bf16_rows;           // plain output as bfloat16 (re, im) pairs
 };
 // The FFT stages run on column pairs (float4 shared-memory accesses, a zero
 // column beside an odd last one). VEC (even rows, 16-byte aligned): the copies
 // and the plain output move pairs too, else single columns (8 bytes).
-// SPLIT: the output is the range table's operand (sp.A), else `out`.
+// LIMBS: the output is the range table's operand (sp.A) in that many BF16 parts of
+// each real number (2 or 3), or `out` (0).
 // (Odd rows took single columns through every stage before: a scan of 51
 // frequencies 67.0 -> 65.8 us, of 201 235.9 -> 233.8.)
-template <bool VEC, bool SPLIT>
+template <bool VEC, int LIMBS>
 __global__ void __launch_bounds__(kFftThreads)
 k_fft_strided(const float2 *__restrict__ in, const float2 *__restrict__ in2, float2 *__restrict__ out,
               int n_in, int I, int ld, FftPlan plan, const float2 *__restrict__ tw_g, int sgn,
@@ -99,7 +99,7 @@ k_fft_strided(const float2 *__restrict__ in, const float2 *__restrict__ in2, flo
 
     // the last FFT stage writes the output rows itself: transform index t
     // goes to output row (t - out_off) mod N when that is below out_rows
-    if constexpr (SPLIT) {
+    if constexpr (LIMBS > 0) {
         // (the pair's second column may be the operand's first padding column,
         // which is zero and stays so)
         const size_t plane = (size_t)sp.batch * sp.Kp;
@@ -109,7 +109,7 @@ k_fft_strided(const float2 *__restrict__ in, const float2 *__restrict__ in2, flo
             if (r < 0) r += N;
             if (r >= out_rows || i0 + 2 * cp >= I) return;
             const float2 v0 = cscale(x0, scale), v1 = cscale(x1, scale);
-            if (sp.limbs == 3) {
+            if constexpr (LIMBS == 3) {
                 __nv_bfloat16 *o = A + (size_t)r * 6 * plane + 2 * cp;
                 float re0 = v0.x, re1 = v1.x, im0 = v0.y, im1 = v1.y;
 #pragma unroll
@@ -318,13 +318,14 @@ cudaError_t launch_fft_strided(const float2 *in, float2 *out, int batch, int n_i
     if (ld < I) return cudaErrorInvalidValue;
     const bool pairs = (I % 2 == 0) && (ld % 2 == 0) && ((uintptr_t)in % 16 == 0) &&
                        ((uintptr_t)in2 % 16 == 0) && (split_A || (uintptr_t)out % 16 == 0);
-    auto kern = split_A ? (pairs ? k_fft_strided<true, true> : k_fft_strided<false, true>)
-                        : (pairs ? k_fft_strided<true, false> : k_fft_strided<false, false>);
+    auto kern = pairs ? k_fft_strided<true, 0> : k_fft_strided<false, 0>;
+    if (split_A && split_limbs == 3) kern = pairs ? k_fft_strided<true, 3> : k_fft_strided<false, 3>;
+    else if (split_A) kern = pairs ? k_fft_strided<true, 2> : k_fft_strided<false, 2>;
     cudaError_t e = allow_dynamic_smem(kern, smem);
     if (e != cudaSuccess) return e;
     dim3 grid((I + kFftIB - 1) / kFftIB, batch);
     // bf16_out: with split_A, the hi planes only; else bfloat16 (re, im) rows
-    const SplitOut sp{(__nv_bfloat16 *)split_A, batch, split_Kp, split_A ? bf16_out : 0, split_limbs,
+    const SplitOut sp{(__nv_bfloat16 *)split_A, batch, split_Kp, split_A ? bf16_out : 0,
                       split_A ? 0 : bf16_out};
     kern<<<grid, kFftThreads, smem, st>>>(in, in2, out, n_in, I, ld, plan, tw, sgn, scale, out_rows, out_off,
                                   sp);
