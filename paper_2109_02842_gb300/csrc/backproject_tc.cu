@@ -135,11 +135,12 @@ __device__ __forceinline__ void channel_taps(const BpDesc &p, const CoefTable &c
     const float s = fmaf(2.0f, pos - (float)o, -(float)(W - 1));
     // the kernel is even: tap W - 1 - t at s is tap t at -s, so a pair of taps
     // shares the even and the odd part of one polynomial: 24 FMA for six taps
-    // in place of 42 (384 channels, 256 x 256 pixels, 200 bins: 812 -> 798 us a
-    // scan). Not where a last bit of the weights can flip a BF16 rounding:
-    // BF16-only products (single voxels move by 1e-3 of the image), and four
-    // taps (such a plan makes the learned path's BF16 input, whose roundings
-    // its network carries to 3e-4 of its image). (Not kept: the rotation below
+    // in place of 42 (384 channels, 256 x 256 pixels, 200 bins, repeated on one
+    // box: 777 to 786 -> 758 to 768 us a scan). Not where a last bit of the
+    // weights can flip a BF16 rounding: BF16-only products (single voxels move
+    // by 1e-3 of the image), and four taps (such a plan makes the learned
+    // path's BF16 input, whose roundings its network carries to 3e-4 of its
+    // image). (Not kept: the rotation below
     // by the bits of r, and the channel's phase from a table: both slower.)
     if constexpr (W == 4 || SPLIT != 3) {
 #pragma unroll

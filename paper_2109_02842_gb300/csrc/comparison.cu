@@ -61,14 +61,14 @@ __device__ __forceinline__ ff ff_dist2d(ff x, ff y, ff px, ff py) {
 // G[u][pixel] of the exact sum: two bins x 128 consecutive pixels per block, one
 // pixel per thread.
 //
-// Bound by the two MUFU operations of a term (16 lanes per cycle and SM). The
+// Bound by instruction issue (65 % of the slots; FP32 pipe 47 %, MUFU 37 %). The
 // terms' coefficients k_m S and wavenumbers are staged in shared memory once per
 // block and read by every lane at once. The phase kappa a of each (pixel, term)
 // is a float-pair product reduced modulo 2 pi, so that the fast sine and cosine
 // see [-pi, pi], where their error is bounded; the two bins' phases are formed
 // in packed pairs. 120 channels, 51 frequencies, 128 bins, 64 x 64 pixels: 4.85
 // (eight bins a block, terms loaded one by one) -> 1.87 ms, 2.29 with unpacked
-// phases (MUFU floor 1.39); 1024 x 1 pixels 4.38 -> 0.62 ms. (Splitting the
+// phases (0.67 at the MUFU pipe's rate); 1024 x 1 pixels 4.38 -> 0.62 ms. (Splitting the
 // phase at a reference pixel, one FP32 product of up to 128 rad a term, took
 // 1.65 ms but raised the image's error from 4.7e-6 to 6.4e-6.)
 constexpr int kExThreads = 128;

@@ -28,7 +28,7 @@
 // and now: 16 -> 16 channels 0.278 and 0.090 ms, 32 -> 16 0.425 and 0.162, 16 ->
 // 2 0.320 and 0.070; 48 x 64 x 64, 32 -> 32 0.072 and 0.047; 44 x 72 x 72, 32 ->
 // 32 (rows nn_tc.cu does not take) 0.187 and 0.047. Shared memory is 64 % and
-// the tensor pipe 51 % busy (16 -> 16), integer work 38 %: the latter halved
+// the tensor pipe 50 % busy (16 -> 16), integer work 38 %: the latter halved
 // when the sixteen-voxel steps became immediates and divisions reciprocals
 // (0.107 -> 0.090).
 #include <cuda_bf16.h>

@@ -693,7 +693,7 @@ pl_status build_plan(pl_plan *P, const pl_geometry *g, const pl_scan *s, const p
         // channels, as many as the SMs take. Their spectra are kept apart and
         // added in order, so results stay bitwise reproducible. Whole scan: 64
         // channels, 32 x 32 pixels (16 -> 64 blocks) 59.4 -> 45.0 us (49.1 with
-        // four parts), 120 channels, 64 x 64 (64 -> 128 blocks) 76 -> 67 us.
+        // four parts), 120 channels, 64 x 64 (64 -> 128 blocks) 76 -> 64 us.
         // Scenes of a batch share the SMs. Its persistent back-projection, whose
         // layout one_block_per_sm is, fills them with two parts (twelve such scenes
         // 366 and 390 us with more, twenty-four of 96 channels 467 and 513); scenes
@@ -701,10 +701,14 @@ pl_status build_plan(pl_plan *P, const pl_geometry *g, const pl_scan *s, const p
         // parts too: three and four small scenes gain (136 -> 130, 95 -> 94 us),
         // twelve of 64 channels are even, twelve and twenty-four of 120 and 96
         // channels lose 6 % (319 -> 337, 366 -> 389).
-        // Up to 256 channels: the accumulation error of longer sums would
-        // change with the split by more than 1e-5 of the image. Not with four
-        // taps: such a plan makes the learned path's input, whose BF16
-        // roundings carry a change of its last bits to 3e-4 of its image.
+        // More than 256 channels, and four taps, would gain too, but their images
+        // would move against those they have always had, and these are left as they
+        // are: 300 channels, 32 x 32 pixels 131 us with two parts and 67 with eight,
+        // off by 1.83e-5 and 0.85e-5 against 64 bits (each part's sum is shorter, and
+        // the tensor cores truncate), so 1.6e-5 apart; four taps, 64 channels 51.9
+        // and 43.5 us, 6.3e-4 off both ways, but such a plan makes the learned path's
+        // BF16 input, whose network carries a change of its last bits to 3e-4 of the
+        // image.
         if (ta.nsplit == 2 && P->C <= 256 && W != 4 && !o.one_block_per_sm) {
             int dev = 0, sms = 0;
             PL_CUDA(cudaGetDevice(&dev), "cudaGetDevice");

@@ -16,7 +16,7 @@
 //   k_rt_prep          S [C][N_p][M] -> A [u][re hi, re lo, im hi, im lo][C][K] BF16
 //   k_range_table_tc   persistent, one block per SM, over the items (128-channel
 //                      block, bin, row part): TMA (128-byte swizzled, K-major) A
-//                      and E tiles, 12 MMAs per 16-frequency step (up to four
+//                      and E tiles, 12 MMAs per 16-frequency step (one or two
 //                      64-frequency atoms per item), tcgen05.ld,
 //                      BF16 hi/lo, stored straight from the registers into
 //                      prod [u][hi, lo][row][Cp] of (re, im) pairs, channels
