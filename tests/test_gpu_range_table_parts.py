@@ -54,7 +54,7 @@ def operand(plan, binding, stage, rows, kp):
 
 @pytest.mark.parametrize("per,n_f,n,n_pad,nx,ext", [
     (128, 129, 64, 128, 24, 0.14), (200, 201, 100, 135, 24, 0.14), (130, 256, 128, 128, 70, 0.45),
-    (64, 192, 270, 360, 24, 0.14), (140, 160, 127, 127, 24, 0.14)])
+    (64, 192, 270, 360, 24, 0.14), (140, 160, 127, 127, 24, 0.14), (65, 193, 100, 256, 148, 0.95)])
 def test_operands_and_table(binding, per, n_f, n, n_pad, nx, ext):
     plan = binding.Plan.from_workload(workload(per, n_f, n, n_pad, nx, ext), block_config=4)
     i = plan.info
@@ -83,3 +83,19 @@ def test_operands_and_table(binding, per, n_f, n, n_pad, nx, ext):
 def test_few_channels_keep_the_nufft(binding, per, n_pad, exact):
     plan = binding.Plan.from_workload(workload(per, 201, 200, n_pad))
     assert plan.info["table_exact"] == exact
+
+
+def test_a_wait_that_runs_out(binding):
+    # (the range table's first stage waits on a barrier nothing completes, for 2 ms)
+    w = workload(64, 160, 200, 256)
+    e = torch.randn((64, 200, 160), dtype=torch.complex64, device="cuda")
+    plan = binding.Plan.from_workload(w, block_config=4, debug_unsatisfiable=2, wait_timeout_us=2000)
+    assert plan.info["table_exact"] == 1
+    plan.execute(e)
+    torch.cuda.synchronize()
+    with pytest.raises(binding.PolylineError) as err:
+        plan.execute(e)
+    assert err.value.status == 8         # PL_ERR_TIMEOUT
+    plan.close()
+    good = binding.Plan.from_workload(w, block_config=4, wait_timeout_us=2000)
+    assert torch.equal(good.execute(e), good.execute(e))
